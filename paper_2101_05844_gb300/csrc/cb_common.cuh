@@ -80,6 +80,20 @@ struct DSched {
     float sp_lr0, sp_lr1;
 };
 
+// Schedule of the Big-M / Active Set loop at global iteration it. Worked out once per iteration by the
+// launch that advances the counter (and wherever the counter is set), and read by the passes: worked out
+// per unit, its divisions and bias corrections were a third of the passes' instructions.
+struct Step {
+    int it;
+    int as_phase;       // 0 Big-M, 1 Active Set
+    int t;              // Active Set local iteration (-1 in Big-M)
+    int b_new;          // slot added at this iteration (-1: none)
+    int nadd_before;    // slots added before this iteration (global, before per-subproblem caps)
+    float lr;
+    float2 ib;                 // Adam's 1 / (1 - b1^n), 1 / (1 - b2^n) of alpha, beta_0, beta_1
+    float2 sib[CB_MAXCUT];     // and of each slot, by its own step count
+};
+
 // Device state. Per-subproblem arrays are [S][NT], [S][NH] or [S][cap][NH].
 struct DState {
     float *lo, *hi;                  // post-activation bounds, layer 0 = input box
@@ -125,15 +139,7 @@ struct DState {
     float *ab, *b0i, *b1i;           // [S][NH] primal-init inner maximisers
     float* arow;                     // [S][NH] ab - b1i (primal-init row values for the col pass)
     int* status;                     // device error word
-};
-
-// Iteration schedule of the Big-M / Active Set loop at global iteration it.
-struct Step {
-    int as_phase;       // 0 Big-M, 1 Active Set
-    int t;              // Active Set local iteration (-1 in Big-M)
-    int b_new;          // slot added at this iteration (-1: none)
-    int nadd_before;    // slots added before this iteration (global, before per-subproblem caps)
-    float lr;
+    Step* step;                      // schedule of the iteration ctr[0] names
 };
 
 __host__ __device__ inline int cb_additions_before(int t, const DSched& d) {
@@ -162,15 +168,38 @@ __host__ __device__ inline int cb_slot_added_at(int b, const DSched& d) {
     return d.omega > 0 ? (b / d.vpa) * d.omega + (b % d.vpa) : b;
 }
 
-__device__ inline Step cb_step(int it, const DSched& d, const float* lr_tab) {
-    Step s;
-    s.lr = it < d.ntab ? lr_tab[it] : d.lr_as_end;
-    if (it < d.TM) {
-        s.as_phase = 0; s.t = -1; s.b_new = -1; s.nadd_before = 0;
-    } else {
-        s.as_phase = 1; s.t = it - d.TM;
-        s.b_new = cb_slot_at(s.t, d);
-        s.nadd_before = cb_additions_before(s.t, d);
-    }
-    return s;
+// 1 / (1 - beta^step), the Adam bias corrections, from a table built in FP64 on the host.
+__device__ __forceinline__ float inv_bias_corr(const float* tab, int ntab, int step, float beta) {
+    return step < ntab ? tab[step] : 1.f / (1.f - powf(beta, (float)step));
 }
+
+// Works out *st.step for iteration `it`: lane b of a warp its slot b, lane 0 the rest.
+__device__ inline void cb_set_step(int it, const DSched& d, const DState& st, int lane) {
+    Step* s = st.step;
+    const int t = it - d.TM;
+    if (lane < CB_MAXCUT) {
+        // a slot's first step is the iteration that adds it (values of slots not yet added are not read)
+        const int n = max(0, t - cb_slot_added_at(lane, d)) + 1;
+        s->sib[lane] = make_float2(inv_bias_corr(st.bc1_tab, d.ntab, n, d.b1), inv_bias_corr(st.bc2_tab, d.ntab, n, d.b2));
+    }
+    if (lane) return;
+    s->it = it;
+    s->as_phase = t >= 0;
+    s->t = t >= 0 ? t : -1;
+    s->b_new = t >= 0 ? cb_slot_at(t, d) : -1;
+    s->nadd_before = t >= 0 ? cb_additions_before(t, d) : 0;
+    s->lr = it < d.ntab ? st.lr_tab[it] : d.lr_as_end;
+    s->ib = make_float2(inv_bias_corr(st.bc1_tab, d.ntab, it + 1, d.b1), inv_bias_corr(st.bc2_tab, d.ntab, it + 1, d.b2));
+}
+
+// The schedule's scalars (no pass writes them) and a slot's bias corrections.
+struct StepNow {
+    int it, as_phase, t, b_new, nadd_before;
+    float lr;
+};
+__device__ __forceinline__ StepNow cb_step(const DState& st) {
+    const Step* s = st.step;
+    return {__ldg(&s->it), __ldg(&s->as_phase), __ldg(&s->t), __ldg(&s->b_new), __ldg(&s->nadd_before), __ldg(&s->lr)};
+}
+__device__ __forceinline__ float2 cb_bias(const DState& st) { return __ldg(&st.step->ib); }
+__device__ __forceinline__ float2 cb_slot_bias(const DState& st, int b) { return __ldg(&st.step->sib[b]); }

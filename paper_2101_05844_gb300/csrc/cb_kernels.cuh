@@ -10,73 +10,22 @@
 // bitset in a register, computed from per-neuron snapshot bytes (Active Set) or per-input
 // thresholds (Saddle Point); see cb_slot_mask and cb_sp_mask.
 #pragma once
-#include "cb_common.cuh"
-#include "cb_walk.cuh"
+#include "cb_dev.cuh"
 
 namespace cb {
 
-// Active Set mask bits of every slot for one (i, j) pair (eq. 3 at binary iterates).
-// zs: bit b = z*_k[i] when slot b was added; xs: bit b = (x*_{k-1}[j] was at its upper bound).
-// With z = 1 the row is all ones; with z = 0 the bit is 1 where the coefficient
-// ((1-z) Lcheck + z Ucheck - x) W is >= 0: W > 0 and x at its lower bound, W < 0 and x at its
-// upper bound, W = 0, or l = u (fixed input, coefficient exactly 0). An input strictly inside its
-// box (interior: layer 0 over an ellipsoid) is at neither end: the bit is z, or 1 where W = 0 or l = u.
-__device__ __forceinline__ unsigned cb_slot_mask(unsigned zs, unsigned xs, bool fixed, float w,
-                                                 bool interior = false) {
-    unsigned xm = fixed ? 0xFFu
-                        : (w > 0.f ? (interior ? 0u : (~xs & 0xFFu)) : (w < 0.f ? (interior ? 0u : xs) : 0xFFu));
-    return zs | xm;
+// Advances the iteration counter ctr[i] (0: Active Set, 1: Saddle Point, 2: primal initialisation)
+// after the launch that completes an iteration, and with the Active Set's the schedule: stream order
+// has every block of that launch done before it, and the next launches read the new values. One warp.
+__global__ void k_advance(DState st, DSched sc, int i) {
+    const int v = st.ctr[i] + 1;
+    __syncwarp();
+    if (threadIdx.x == 0) st.ctr[i] = v;
+    if (i == 0) cb_set_step(v, sc, st, threadIdx.x);
 }
 
-// Saddle Point oracle bit, eq. (3) with continuous (x, z), in the threshold form: W > 0 ->
-// z (u - l) >= x - l, W < 0 -> z (u - l) >= u - x (eq. 3 with the sign of W multiplied out), i.e.
-// z >= tau for tau = (x - l) / (u - l), resp. (u - x) / (u - l); W = 0 or l = u -> 1 (fixed inputs
-// carry thresholds of -inf). The thresholds are cb_tau_up's, so each float32 compare is exact.
-__device__ __forceinline__ bool cb_sp_mask(float z, float tp, float tn, float w) {
-    return w > 0.f ? (z >= tp) : (w < 0.f ? (z >= tn) : true);
-}
-
-// The smallest float32 at or above the real quotient (a - b) / (hi - lo), for float32 a, b, lo <
-// hi: the differences are exact in float64 (float32 operands whose magnitudes lie within 2^28 of
-// each other), the quotient is rounded up in float64 and again to float32. Rounding up twice
-// gives the float32 rounding up of the real quotient (a float32 is a float64), so for every
-// float32 z, z >= tau (real) exactly when z >= this value: the mask decision of eq. (3) is exact.
-__device__ __forceinline__ float cb_tau_up(float a, float b, float lo, float hi) {
-    return __double2float_ru(__ddiv_ru((double)a - (double)b, (double)hi - (double)lo));
-}
-
-// Block-to-segment lookup for launches that cover several layers.
-struct Segs {
-    int n;
-    int layer[CB_MAXL];   // 0-based layer index
-    int start[CB_MAXL + 1];
-};
-__device__ __forceinline__ int seg_of(const Segs& sg, int blk) {
-    int q = 0;
-    while (q + 1 < sg.n && blk >= sg.start[q + 1]) ++q;
-    return q;
-}
-
-// Advances the iteration counter ctr[i] (0: Active Set, 1: Saddle Point, 2: primal
-// initialisation) after the launch that completes an iteration: stream order has every block of
-// that launch done before it, and the next launches read the new value.
-__global__ void k_advance(int* ctr, int i) { ctr[i] += 1; }
-
-// 1 / (1 - beta^step), the Adam bias corrections, from a table built in FP64 on the host.
-__device__ __forceinline__ float inv_bias_corr(const float* tab, int ntab, int step, float beta) {
-    return step < ntab ? tab[step] : 1.f / (1.f - powf(beta, (float)step));
-}
-
-// One projected Adam ascent step (Kingma and Ba) of a dual variable: returns the new value and
-// updates the moments. Fast reciprocal square root and division (a few float32 ulps).
-__device__ __forceinline__ float adam_step(float th, float& m, float& v, float g, float lr, float ibc1,
-                                           float ibc2, const DSched& sc) {
-    m = sc.b1 * m + sc.omb1 * g;
-    v = sc.b2 * v + sc.omb2 * g * g;
-    const float mh = m * ibc1, vh = v * ibc2;
-    const float sq = vh > 0.f ? vh * rsqrtf(vh) : 0.f;
-    return fmaxf(th + lr * __fdividef(mh, sq + sc.eps), 0.f);
-}
+// The schedule of the iteration the counter names, after the host has set it. One warp.
+__global__ void k_set_step(DState st, DSched sc) { cb_set_step(st.ctr[0], sc, st, threadIdx.x); }
 
 // ------------------------------------------------------------------------- interval bounds
 // Interval propagation for hidden layer L (App. E): lhat = W+ l + W- u + b, uhat = W+ u + W- l + b
@@ -148,8 +97,10 @@ __global__ void k_ibp(DNet net, DState st, int li, const signed char* splits) {
     }
 }
 
-__global__ void k_fill(double* p, size_t n, double v) {
-    for (size_t u = blockIdx.x * (size_t)blockDim.x + threadIdx.x; u < n; u += (size_t)gridDim.x * blockDim.x) p[u] = v;
+// A batch's start: no best bound yet, the schedule of iteration 0 (the counters have been cleared).
+__global__ void k_start(DState st, DSched sc, int S) {
+    if (blockIdx.x == 0 && threadIdx.x < 32) cb_set_step(0, sc, st, threadIdx.x);
+    for (int u = blockIdx.x * blockDim.x + threadIdx.x; u < S; u += gridDim.x * blockDim.x) st.best[u] = -INFINITY;
 }
 __global__ void k_fill_int(int* p, size_t n, int v) {
     for (size_t u = blockIdx.x * (size_t)blockDim.x + threadIdx.x; u < n; u += (size_t)gridDim.x * blockDim.x) p[u] = v;
@@ -260,7 +211,7 @@ __global__ void k_reduce(DNet net, DState st, int precision, double* out, int ke
 // price caps of eq. (16).
 __global__ void k_sp_convert_elem(DNet net, DState st, DSched sc, float c_alpha, float c_beta) {
     const size_t n = (size_t)net.S * net.NH;
-    const Step sp = cb_step(st.ctr[0], sc, st.lr_tab);
+    const StepNow sp = cb_step(st);
     for (size_t u = blockIdx.x * (size_t)blockDim.x + threadIdx.x; u < n; u += (size_t)gridDim.x * blockDim.x) {
         const int s = (int)(u / net.NH), hh = (int)(u - (size_t)s * net.NH);
         int li = 0;

@@ -27,14 +27,6 @@ namespace cb {
 
 #define CB_MAXTAP 9
 
-struct TSegs {
-    int n;
-    int layer[CB_MAXL];
-    int start[CB_MAXL + 1];   // first block of each segment
-    int T[CB_MAXL];           // team size (1, 2, 4, 8, 16 or 32)
-    const int* perm[CB_MAXL]; // col pass of a strided conv: unit order -> input index (or null)
-};
-
 template <class Fn>
 __device__ __forceinline__ void col_walk_team(const DLayer& L, int j, int lane, int T, Fn fn) {
     if (L.kind == 0) {
@@ -94,70 +86,6 @@ __device__ __forceinline__ void col_walk_team(const DLayer& L, int j, int lane, 
     }
 }
 
-__device__ __forceinline__ float team_sum(float v, int T) {
-    for (int o = T >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
-// ---------------------------------------------------------------- Active Set walks
-// Group and base position of row-pass unit i (output neuron i of layer L).
-__device__ __forceinline__ void row_group(const DLayer& L, int i, int& g, int& base) {
-    if (L.kind == 0) {
-        g = i;
-        base = 0;
-        return;
-    }
-    const int hw = L.ho * L.wo;
-    const int co = i / hw, rem = i - co * hw;
-    const int oy = rem / L.wo, ox = rem - oy * L.wo;
-    g = co;
-    base = oy * L.st * L.Wp + ox * L.st;
-}
-
-// Group and base position of col-pass unit j (input neuron j of layer L).
-__device__ __forceinline__ void col_group(const DLayer& L, int j, int& g, int& base) {
-    if (L.kind == 0) {
-        g = j;
-        base = 0;
-        return;
-    }
-    const int hw = L.hi * L.wi;
-    const int c = j / hw, rem = j - c * hw;
-    const int y = rem / L.wi, x = rem - y * L.wi;
-    const int ty = y + L.pd, tx = x + L.pd;
-    const int Y0 = ty / L.st, X0 = tx / L.st;
-    const int py = ty - Y0 * L.st, px = tx - X0 * L.st;
-    g = (c * L.st + py) * L.st + px;
-    base = (Y0 + L.hl) * L.Wpo + X0 + L.wl;
-}
-
-// Record position of input neuron j (row-pass input records) and output neuron i (col-pass
-// output records) of layer L.
-__device__ __forceinline__ int xin_pos(const DLayer& L, int j) {
-    if (L.kind == 0) return j;
-    const int hw = L.hi * L.wi;
-    const int c = j / hw, rem = j - c * hw;
-    const int y = rem / L.wi, x = rem - y * L.wi;
-    return (c * L.Hp + y + L.pd) * L.Wp + x + L.pd;
-}
-__device__ __forceinline__ int arec_pos(const DLayer& L, int i) {
-    if (L.kind == 0) return i;
-    const int hw = L.ho * L.wo;
-    const int co = i / hw, rem = i - co * hw;
-    const int oy = rem / L.wo, ox = rem - oy * L.wo;
-    return (co * L.Hpo + oy + L.hl) * L.Wpo + ox + L.wl;
-}
-
-// Output records of layer L for subproblem s: RS / 4 planes of float4, plane q holding entries
-// 4q .. 4q + 3 of every position, so that lanes reading neighbouring positions read one
-// contiguous run per plane.
-__device__ __forceinline__ float4* arec_planes(const DNet& net, const DState& st, const DLayer& L, int s) {
-    return reinterpret_cast<float4*>(st.arec + (size_t)s * net.AT + L.ao);
-}
-__device__ __forceinline__ float* arec_entry(const DNet& net, const DState& st, const DLayer& L, int s, int p, int e) {
-    return reinterpret_cast<float*>(arec_planes(net, st, L, s) + (size_t)(e >> 2) * L.apos + p) + (e & 3);
-}
-
 // The first NV entries of the record at q (planes apos apart).
 template <int NV>
 __device__ __forceinline__ void load_rec(const float4* q, int apos, float (&v)[12]) {
@@ -165,20 +93,6 @@ __device__ __forceinline__ void load_rec(const float4* q, int apos, float (&v)[1
     v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
     if (NV > 4) { const float4 b = q[apos]; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w; }
     if (NV > 8) { const float4 c = q[2 * apos]; v[8] = c.x; v[9] = c.y; v[10] = c.z; v[11] = c.w; }
-}
-
-// Records of the float32 slot row sums (k_slot_sums_t below): per input {l, u, p bits | q bits
-// << 8} in the first Saddle Point input plane, which Active Set leaves unused.
-__device__ __forceinline__ float4* slot_rec_plane(const DNet& net, const DState& st, const DLayer& L, int s) {
-    return st.spin + (size_t)s * net.XT + (size_t)L.xo;
-}
-// The record of an input with box [lo, hi] and snapshot bits xs (bit b: at its upper end when slot b
-// was added); a fixed input (lo = hi) is selected by every mask, an interior one (layer 0 over an
-// ellipsoid) by none: its bit is z alone.
-__device__ __forceinline__ float4 slot_rec(float lo, float hi, unsigned xs, bool fixed, bool interior) {
-    const unsigned fxm = fixed ? 0xFFu : 0u;
-    const unsigned pm = (interior ? 0u : (~xs & 0xFFu)) | fxm, qm = (interior ? 0u : (xs & 0xFFu)) | fxm;
-    return make_float4(lo, hi, __uint_as_float(pm | (qm << 8)), 0.f);
 }
 
 // B taps of a lane's stride T starting at t (taps at or past tb read as {0, +0.f}: a zero weight
@@ -247,9 +161,7 @@ __device__ __forceinline__ int div_stride(int a, int st) { return st == 1 ? a : 
 template <int NS>
 __device__ __forceinline__ void as_colA_body(const DNet& net, const DState& st, const DSched& sc, const DLayer& L,
                                              int k, bool valid, int s, int j, int lane, int T, int mode) {
-    const int m = k - 1;
-    const Step sp = cb_step(st.ctr[0], sc, st.lr_tab);
-    const size_t NT = net.NT, NH = net.NH, cap = net.cap;
+    const StepNow sp = cb_step(st);
     float acc = 0.f, Pp[NS > 0 ? NS : 1], Pn[NS > 0 ? NS : 1];
 #pragma unroll
     for (int b = 0; b < NS; ++b) Pp[b] = Pn[b] = 0.f;
@@ -290,22 +202,11 @@ __device__ __forceinline__ void as_colA_body(const DNet& net, const DState& st, 
         }
     }
     if (!valid || lane != 0) return;
-    const bool want_terms = mode != 2;
-    const int cap_s = st.caps[s];
-    const int nsl = min(sp.nadd_before, cap_s);
-    const int bo = sp.nadd_before & 1;
-    const bool add_iter = (mode != 1) && sp.b_new >= 0;
-    const bool add = add_iter && sp.b_new < cap_s;
-    const size_t xo = (size_t)s * NT + L.in_off + j;
-    const float lo = st.lo[xo], hi = st.hi[xo];
-    const unsigned xs = st.xsnap[bo][xo];
-    const bool fixed = st.efix[xo];
-    const unsigned fxm = fixed ? 0xFFu : 0u;
+    const ColState<NS> c = as_colA_load<NS>(net, st, sp, L, k, s, j, mode);
     float f;
     if (k <= net.n - 1) {
-        // an interior input (layer 0 over an ellipsoid) is at neither end of its box: eq. (3) gives z
-        const bool interior = net.ball && L.in_off == 0;
-        const unsigned pm = (interior ? 0u : ((~xs) & 0xFFu)) | fxm, qm = (interior ? 0u : xs) | fxm;
+        unsigned pm, qm;
+        slot_bits(net, L, c.xs, c.fixed, pm, qm);
         f = acc;
 #pragma unroll
         for (int b = 0; b < NS; ++b) {
@@ -315,59 +216,7 @@ __device__ __forceinline__ void as_colA_body(const DNet& net, const DState& st, 
     } else {
         f = -net.Wout[(size_t)s * L.n_in + j];
     }
-    double term = 0.0;
-    if (m >= 1) {
-        const size_t h = (size_t)s * NH + L.h_in + j;
-        const size_t hs = (size_t)s * cap * NH + L.h_in + j;
-        float sb = 0.f, gk = st.beta0[h] * st.uhat[h] + st.beta1[h] * st.lhat[h];
-        double cterm = 0.0;
-        // all slot loads first (NS >= nsl), then the sums in slot order
-        float bbv[NS > 0 ? NS : 1], kpv[NS > 0 ? NS : 1], lmv[NS > 0 ? NS : 1];
-#pragma unroll
-        for (int b = 0; b < NS; ++b) {
-            bbv[b] = kpv[b] = lmv[b] = 0.f;
-            if (b < nsl) {
-                bbv[b] = st.bs[hs + (size_t)b * NH];
-                kpv[b] = st.kap[hs + (size_t)b * NH];
-                if (want_terms) lmv[b] = st.lam[hs + (size_t)b * NH];
-            }
-        }
-#pragma unroll
-        for (int b = 0; b < NS; ++b)
-            if (b < nsl) {
-                sb += bbv[b];
-                gk += bbv[b] * kpv[b];
-                if (want_terms) cterm += (double)bbv[b] * lmv[b];
-            }
-        f += st.alpha[h] - st.beta0[h] - st.beta1[h] - sb;
-        const bool z = gk >= 0.f;
-        st.zcur[h] = z;
-        if (want_terms) {
-            const float bm = net.L[m - 1].b[j];
-            term = (double)bm * st.alpha[h] + (double)st.beta1[h] * ((double)st.lhat[h] - bm) + cterm -
-                   (z ? (double)gk : 0.0);
-        }
-        if (add_iter) {
-            const unsigned zs_old = st.zsnap[bo][h];
-            st.zsnap[bo ^ 1][h] = (uint8_t)(zs_old | ((add && z) ? (1u << sp.b_new) : 0u));
-        }
-    }
-    const bool up = f >= 0.f;
-    const float xv = up ? hi : lo;
-    st.xval[xo] = xv;
-    st.fval[xo] = f;
-    if (want_terms) st.terms[xo] = term - (double)f * xv;
-    unsigned xs_new = xs;
-    if (add_iter) {
-        xs_new = xs | ((add && up) ? (1u << sp.b_new) : 0u);
-        st.xsnap[bo ^ 1][xo] = (uint8_t)xs_new;
-    }
-    if (k <= net.n - 1) {
-        const unsigned mpos = ((~xs_new) & 0xFFu) | fxm, mneg = (xs_new & 0xFFu) | fxm;
-        // row-pass input record: x* and the slot masks p_b (bits 0-7) and q_b (bits 8-15)
-        reinterpret_cast<float2*>(st.xin + (size_t)s * net.XT + L.xo)[xin_pos(L, j)] =
-            make_float2(xv, __uint_as_float(mpos | (mneg << 8)));
-    }
+    as_colA_unit<NS>(net, st, sp, L, k, s, j, f, c, mode);
 }
 
 // Floats per thread of the BF16 col pass's prefetch (as_colA_tc): the W+ and W- products of slot 0
@@ -383,7 +232,7 @@ __device__ __forceinline__ void as_colA_tc(const DNet& net, const DState& st, co
                                            int k, bool valid, int s, int j, int mode, TcStage* stg, TcPos tp,
                                            float* buf) {
     const int m = k - 1;
-    const Step sp = cb_step(st.ctr[0], sc, st.lr_tab);
+    const StepNow sp = cb_step(st);
     const size_t NT = net.NT, NH = net.NH, cap = net.cap;
     float* my = buf + threadIdx.x;
     auto at = [&](int v) -> float& { return my[v * CB_THREADS]; };
@@ -562,7 +411,7 @@ __global__ void __launch_bounds__(CB_BALL_THREADS) k_ball_x0(DNet net, DState st
         st.terms[base] = -red[1][0] - nrm;
         st.bnrm[s] = nrm;
     }
-    float2* rec = reinterpret_cast<float2*>(st.xin + (size_t)s * net.XT + L.xo);
+    float2* rec = xin_recs(net, st, L, s);
     for (int j = threadIdx.x; j < L.n_in; j += CB_BALL_THREADS) {
         const size_t xo = base + j;
         const float lo = st.lo[xo], hi = st.hi[xo];
@@ -652,7 +501,7 @@ __global__ void __launch_bounds__(CB_THREADS, 4) k_as_colA_t(DNet net, DState st
         for (int e = 0; e < 2 * (net.cap + 1); ++e) stage_at(stage, e) = 0;
     TcStage* stg = staged ? &stage : nullptr;
     const int j = (valid && sg.perm[q]) ? sg.perm[q][o] : o;
-    const Step sp = cb_step(st.ctr[0], sc, st.lr_tab);
+    const StepNow sp = cb_step(st);
     const int ns = min(sp.nadd_before, sc.maxcut);
     if constexpr (TC) {
         extern __shared__ float colA_buf[];
@@ -711,7 +560,7 @@ __global__ void __launch_bounds__(CB_THREADS, 4) k_as_colA_t(DNet net, DState st
 // in exact arithmetic.
 template <int NS, bool ADD>
 __device__ __forceinline__ void as_rowB_body(const DNet& net, const DState& st, const DSched& sc, const DLayer& L,
-                                             int li, bool valid, int s, int i, int lane, int T, const Step& sp, int it) {
+                                             int li, bool valid, int s, int i, int lane, int T, const StepNow& sp) {
     const size_t NT = net.NT, NH = net.NH, cap = net.cap;
     const int cap_s = valid ? st.caps[s] : 0;
     const int newb = (ADD && sp.b_new < cap_s) ? sp.b_new : -1;
@@ -725,7 +574,7 @@ __device__ __forceinline__ void as_rowB_body(const DNet& net, const DState& st, 
     if (valid) {
         int g, base;
         row_group(L, i, g, base);
-        const float2* xb = reinterpret_cast<const float2*>(st.xin + (size_t)s * net.XT + L.xo) + base;
+        const float2* xb = xin_recs(net, st, L, s) + base;
         const int t0 = L.rgrp[2 * g], t1 = L.rgrp[2 * g + 1], t2 = L.rgrp[2 * g + 2];
         // positive taps take the slot masks p_b (bits 0-7), negative taps q_b (bits 8-15)
         constexpr int B = 6;   // six taps and records in flight fit 64 registers
@@ -755,6 +604,12 @@ __device__ __forceinline__ void as_rowB_body(const DNet& net, const DState& st, 
 #pragma unroll
         for (int b = 0; b < NS; ++b) acc[b] = team_sum(acc[b], T);
     }
+    if (T == 1) {
+        if (!valid) return;
+        RowState<NS> r = as_rowB_load<NS, ADD, false>(net, st, L, s, i, sp);
+        as_rowB_unit<NS, ADD, false>(net, st, sc, L, s, i, sp, acc0, acc, r);
+        return;
+    }
     // epilogue: the team's lanes share the Adam updates (variable v = alpha, beta_0, beta_1, then
     // the slots), each lane handling v = lane, lane + T, ...
     const int nsl = min(sp.nadd_before + (sp.b_new >= 0 ? 1 : 0), cap_s);
@@ -768,84 +623,15 @@ __device__ __forceinline__ void as_rowB_body(const DNet& net, const DState& st, 
         const int ap = arec_pos(L, i);
         // the col pass's record entry e of this row
         auto put = [&](int e, float v) { *arec_entry(net, st, L, s, ap, e) = v; };
-        if (T == 1) {
-            // one lane per unit: every load first, so that they are in flight together (the state
-            // arrays may alias as far as the compiler knows, so it would not hoist them itself)
-            float th3[3] = {st.alpha[h], st.beta0[h], st.beta1[h]};
-            float m3[3] = {st.ma[h], st.m0[h], st.m1[h]};
-            float v3[3] = {st.va[h], st.v0[h], st.v1[h]};
-            const float uh = st.uhat[h], lh = st.lhat[h];
-            const int step = it + 1;
-            const float ib1 = inv_bias_corr(st.bc1_tab, sc.ntab, step, sc.b1);
-            const float ib2 = inv_bias_corr(st.bc2_tab, sc.ntab, step, sc.b2);
-            const float g3[3] = {xhat - x, x - z * uh, x - xhat + (1.f - z) * lh};
-#pragma unroll
-            for (int v = 0; v < 3; ++v) th3[v] = adam_step(th3[v], m3[v], v3[v], g3[v], sp.lr, ib1, ib2, sc);
-            st.alpha[h] = th3[0]; st.beta0[h] = th3[1]; st.beta1[h] = th3[2];
-            st.ma[h] = m3[0]; st.m0[h] = m3[1]; st.m1[h] = m3[2];
-            st.va[h] = v3[0]; st.v0[h] = v3[1]; st.v1[h] = v3[2];
-            contrib = th3[2] - th3[0];
-            // the slots in pairs: a pair's loads first, then its updates (larger groups spill)
-#pragma unroll
-            for (int b0 = 0; b0 < NS; b0 += 2) {
-                float bsv[2], msv[2], vsv[2], lamv[2], kapv[2];
-#pragma unroll
-                for (int q = 0; q < 2; ++q) {
-                    const int b = b0 + q;
-                    bsv[q] = msv[q] = vsv[q] = lamv[q] = kapv[q] = 0.f;
-                    if (b < NS && b < nsl) {
-                        const size_t hs = hs0 + (size_t)b * NH;
-                        bsv[q] = st.bs[hs];
-                        msv[q] = st.ms[hs];
-                        vsv[q] = st.vs[hs];
-                        if (!(ADD && b == newb)) {
-                            lamv[q] = st.lam[hs];
-                            kapv[q] = st.kap[hs];
-                        }
-                    }
-                }
-#pragma unroll
-                for (int q = 0; q < 2; ++q) {
-                    const int b = b0 + q;
-                    if (b >= NS) continue;
-                    if (b >= nsl) {
-                        put(1 + b, 0.f);
-                        continue;
-                    }
-                    const size_t hs = hs0 + (size_t)b * NH;
-                    const bool zb = (zs >> b) & 1u;
-                    float lam = lamv[q], kap = kapv[q];
-                    if (ADD && b == newb) {
-                        const float lzh = st.lz[h];
-                        lam = zb ? lzh : acc[b];
-                        // kappa = lambda + sum W (1 - I) Ucheck + b: W x* + b at box vertices; over
-                        // interior inputs (layer 0, ellipsoid) the z = 0 mask holds fixed inputs only
-                        kap = zb ? lzh + bi : (net.ball && L.in_off == 0 ? st.uz[h] + bi : xhat);
-                        st.lam[hs] = lam;
-                        st.kap[hs] = kap;
-                    }
-                    const float prod = zb ? acc0 : acc[b];
-                    const float gb = x - prod + lam * (1.f - z) - z * (kap - lam);
-                    const int sstep = sp.t - cb_slot_added_at(b, sc) + 1;
-                    const float nv = adam_step(bsv[q], msv[q], vsv[q], gb, sp.lr,
-                                               inv_bias_corr(st.bc1_tab, sc.ntab, sstep, sc.b1),
-                                               inv_bias_corr(st.bc2_tab, sc.ntab, sstep, sc.b2), sc);
-                    st.bs[hs] = nv; st.ms[hs] = msv[q]; st.vs[hs] = vsv[q];
-                    if (zb) contrib += nv;
-                    put(1 + b, zb ? 0.f : nv);
-                }
-            }
-        } else
         for (int v = lane; v < 3 + NS; v += T) {
             if (v < 3) {
                 float* th = v == 0 ? st.alpha : (v == 1 ? st.beta0 : st.beta1);
                 float* mm = v == 0 ? st.ma : (v == 1 ? st.m0 : st.m1);
                 float* vv = v == 0 ? st.va : (v == 1 ? st.v0 : st.v1);
                 const float g = v == 0 ? xhat - x : (v == 1 ? x - z * st.uhat[h] : x - xhat + (1.f - z) * st.lhat[h]);
-                const int step = it + 1;
+                const float2 ib = cb_bias(st);
                 float m = mm[h], w2 = vv[h];
-                const float nv = adam_step(th[h], m, w2, g, sp.lr, inv_bias_corr(st.bc1_tab, sc.ntab, step, sc.b1),
-                                           inv_bias_corr(st.bc2_tab, sc.ntab, step, sc.b2), sc);
+                const float nv = adam_step(th[h], m, w2, g, sp.lr, ib.x, ib.y, sc);
                 th[h] = nv; mm[h] = m; vv[h] = w2;
                 if (v == 0) contrib -= nv;
                 if (v == 2) contrib += nv;
@@ -871,17 +657,16 @@ __device__ __forceinline__ void as_rowB_body(const DNet& net, const DState& st, 
                 }
                 const float prod = zb ? acc0 : ab;
                 const float gb = x - prod + lam * (1.f - z) - z * (kap - lam);
-                const int sstep = sp.t - cb_slot_added_at(b, sc) + 1;
+                const float2 sib = cb_slot_bias(st, b);
                 float m = st.ms[hs], w2 = st.vs[hs];
-                const float nv = adam_step(st.bs[hs], m, w2, gb, sp.lr, inv_bias_corr(st.bc1_tab, sc.ntab, sstep, sc.b1),
-                                           inv_bias_corr(st.bc2_tab, sc.ntab, sstep, sc.b2), sc);
+                const float nv = adam_step(st.bs[hs], m, w2, gb, sp.lr, sib.x, sib.y, sc);
                 st.bs[hs] = nv; st.ms[hs] = m; st.vs[hs] = w2;
                 if (zb) contrib += nv;
                 put(1 + b, zb ? 0.f : nv);
             }
         }
     }
-    if (T > 1) contrib = team_sum(contrib, T);
+    contrib = team_sum(contrib, T);
     if (valid && lane == 0) *arec_entry(net, st, L, s, arec_pos(L, i), 0) = contrib;
 }
 
@@ -896,7 +681,7 @@ __host__ __device__ constexpr int rowB_tc_vals(int cap) { return 13 + 6 * cap; }
 // memory's rate rather than its latency.
 template <int NS, bool ADD>
 __device__ __forceinline__ void as_rowB_tc(const DNet& net, const DState& st, const DSched& sc, const DLayer& L,
-                                           int li, bool valid, int s, int i, const Step& sp, int it, TcStage* stg,
+                                           int li, bool valid, int s, int i, const StepNow& sp, TcStage* stg,
                                            float* buf) {
     const size_t NT = net.NT, NH = net.NH, cap = net.cap;
     const int cap_s = valid ? st.caps[s] : 0;
@@ -966,15 +751,13 @@ __device__ __forceinline__ void as_rowB_tc(const DNet& net, const DState& st, co
                 reinterpret_cast<__nv_bfloat16*>(B.R)[((long long)e * net.S + s) * B.PR + roff] = __float2bfloat16_rn(v);
             }
         };
-        const int step = it + 1;
-        const float ib1 = inv_bias_corr(st.bc1_tab, sc.ntab, step, sc.b1);
-        const float ib2 = inv_bias_corr(st.bc2_tab, sc.ntab, step, sc.b2);
+        const float2 ib = cb_bias(st);
         const float g3[3] = {xhat - x, x - z * at(V_UH), x - xhat + (1.f - z) * at(V_LH)};
         float th3[3];
 #pragma unroll
         for (int v = 0; v < 3; ++v) {
             float m = at(V_M + v), w2 = at(V_V + v);
-            th3[v] = adam_step(at(V_TH + v), m, w2, g3[v], sp.lr, ib1, ib2, sc);
+            th3[v] = adam_step(at(V_TH + v), m, w2, g3[v], sp.lr, ib.x, ib.y, sc);
             at(V_M + v) = m;
             at(V_V + v) = w2;
         }
@@ -1003,11 +786,9 @@ __device__ __forceinline__ void as_rowB_tc(const DNet& net, const DState& st, co
             }
             const float prod = zb ? acc0 : accb;
             const float gb = x - prod + lam * (1.f - z) - z * (kap - lam);
-            const int sstep = sp.t - cb_slot_added_at(b, sc) + 1;
+            const float2 sib = cb_slot_bias(st, b);
             float m = at(V_SL + 5 * b + 1), w2 = at(V_SL + 5 * b + 2);
-            const float nv = adam_step(at(V_SL + 5 * b), m, w2, gb, sp.lr,
-                                       inv_bias_corr(st.bc1_tab, sc.ntab, sstep, sc.b1),
-                                       inv_bias_corr(st.bc2_tab, sc.ntab, sstep, sc.b2), sc);
+            const float nv = adam_step(at(V_SL + 5 * b), m, w2, gb, sp.lr, sib.x, sib.y, sc);
             st.bs[hs] = nv; st.ms[hs] = m; st.vs[hs] = w2;
             if (zb) contrib += nv;
             put(1 + b, zb ? 0.f : nv);
@@ -1036,8 +817,7 @@ __global__ void __launch_bounds__(CB_THREADS, 4) k_as_rowB_t(DNet net, DState st
         valid = i >= 0;
         i = valid ? i : 0;
     }
-    const int it = st.ctr[0];
-    const Step sp = cb_step(it, sc, st.lr_tab);
+    const StepNow sp = cb_step(st);
     const int ns = min(sp.nadd_before + (sp.b_new >= 0 ? 1 : 0), sc.maxcut);
     if (staged)   // zeros stay where the tile has no unit (channel padding)
         for (int e = 0; e <= ns; ++e) stage_at(stage, e) = 0;
@@ -1047,50 +827,50 @@ __global__ void __launch_bounds__(CB_THREADS, 4) k_as_rowB_t(DNet net, DState st
         extern __shared__ float rowB_buf[];
         if (sp.b_new >= 0) {
             switch (ns) {
-                case 1: as_rowB_tc<1, true>(net, st, sc, L, li, valid, s, i, sp, it, stg, rowB_buf); break;
-                case 2: as_rowB_tc<2, true>(net, st, sc, L, li, valid, s, i, sp, it, stg, rowB_buf); break;
-                case 3: as_rowB_tc<3, true>(net, st, sc, L, li, valid, s, i, sp, it, stg, rowB_buf); break;
-                case 4: as_rowB_tc<4, true>(net, st, sc, L, li, valid, s, i, sp, it, stg, rowB_buf); break;
-                case 5: as_rowB_tc<5, true>(net, st, sc, L, li, valid, s, i, sp, it, stg, rowB_buf); break;
-                case 6: as_rowB_tc<6, true>(net, st, sc, L, li, valid, s, i, sp, it, stg, rowB_buf); break;
-                case 7: as_rowB_tc<7, true>(net, st, sc, L, li, valid, s, i, sp, it, stg, rowB_buf); break;
-                default: as_rowB_tc<8, true>(net, st, sc, L, li, valid, s, i, sp, it, stg, rowB_buf); break;
+                case 1: as_rowB_tc<1, true>(net, st, sc, L, li, valid, s, i, sp, stg, rowB_buf); break;
+                case 2: as_rowB_tc<2, true>(net, st, sc, L, li, valid, s, i, sp, stg, rowB_buf); break;
+                case 3: as_rowB_tc<3, true>(net, st, sc, L, li, valid, s, i, sp, stg, rowB_buf); break;
+                case 4: as_rowB_tc<4, true>(net, st, sc, L, li, valid, s, i, sp, stg, rowB_buf); break;
+                case 5: as_rowB_tc<5, true>(net, st, sc, L, li, valid, s, i, sp, stg, rowB_buf); break;
+                case 6: as_rowB_tc<6, true>(net, st, sc, L, li, valid, s, i, sp, stg, rowB_buf); break;
+                case 7: as_rowB_tc<7, true>(net, st, sc, L, li, valid, s, i, sp, stg, rowB_buf); break;
+                default: as_rowB_tc<8, true>(net, st, sc, L, li, valid, s, i, sp, stg, rowB_buf); break;
             }
         } else {
             switch (ns) {
-                case 0: as_rowB_tc<0, false>(net, st, sc, L, li, valid, s, i, sp, it, stg, rowB_buf); break;
-                case 1: as_rowB_tc<1, false>(net, st, sc, L, li, valid, s, i, sp, it, stg, rowB_buf); break;
-                case 2: as_rowB_tc<2, false>(net, st, sc, L, li, valid, s, i, sp, it, stg, rowB_buf); break;
-                case 3: as_rowB_tc<3, false>(net, st, sc, L, li, valid, s, i, sp, it, stg, rowB_buf); break;
-                case 4: as_rowB_tc<4, false>(net, st, sc, L, li, valid, s, i, sp, it, stg, rowB_buf); break;
-                case 5: as_rowB_tc<5, false>(net, st, sc, L, li, valid, s, i, sp, it, stg, rowB_buf); break;
-                case 6: as_rowB_tc<6, false>(net, st, sc, L, li, valid, s, i, sp, it, stg, rowB_buf); break;
-                case 7: as_rowB_tc<7, false>(net, st, sc, L, li, valid, s, i, sp, it, stg, rowB_buf); break;
-                default: as_rowB_tc<8, false>(net, st, sc, L, li, valid, s, i, sp, it, stg, rowB_buf); break;
+                case 0: as_rowB_tc<0, false>(net, st, sc, L, li, valid, s, i, sp, stg, rowB_buf); break;
+                case 1: as_rowB_tc<1, false>(net, st, sc, L, li, valid, s, i, sp, stg, rowB_buf); break;
+                case 2: as_rowB_tc<2, false>(net, st, sc, L, li, valid, s, i, sp, stg, rowB_buf); break;
+                case 3: as_rowB_tc<3, false>(net, st, sc, L, li, valid, s, i, sp, stg, rowB_buf); break;
+                case 4: as_rowB_tc<4, false>(net, st, sc, L, li, valid, s, i, sp, stg, rowB_buf); break;
+                case 5: as_rowB_tc<5, false>(net, st, sc, L, li, valid, s, i, sp, stg, rowB_buf); break;
+                case 6: as_rowB_tc<6, false>(net, st, sc, L, li, valid, s, i, sp, stg, rowB_buf); break;
+                case 7: as_rowB_tc<7, false>(net, st, sc, L, li, valid, s, i, sp, stg, rowB_buf); break;
+                default: as_rowB_tc<8, false>(net, st, sc, L, li, valid, s, i, sp, stg, rowB_buf); break;
             }
         }
     } else if (sp.b_new >= 0) {
         switch (ns) {
-            case 1: as_rowB_body<1, true>(net, st, sc, L, li, valid, s, i, lane, T, sp, it); break;
-            case 2: as_rowB_body<2, true>(net, st, sc, L, li, valid, s, i, lane, T, sp, it); break;
-            case 3: as_rowB_body<3, true>(net, st, sc, L, li, valid, s, i, lane, T, sp, it); break;
-            case 4: as_rowB_body<4, true>(net, st, sc, L, li, valid, s, i, lane, T, sp, it); break;
-            case 5: as_rowB_body<5, true>(net, st, sc, L, li, valid, s, i, lane, T, sp, it); break;
-            case 6: as_rowB_body<6, true>(net, st, sc, L, li, valid, s, i, lane, T, sp, it); break;
-            case 7: as_rowB_body<7, true>(net, st, sc, L, li, valid, s, i, lane, T, sp, it); break;
-            default: as_rowB_body<8, true>(net, st, sc, L, li, valid, s, i, lane, T, sp, it); break;
+            case 1: as_rowB_body<1, true>(net, st, sc, L, li, valid, s, i, lane, T, sp); break;
+            case 2: as_rowB_body<2, true>(net, st, sc, L, li, valid, s, i, lane, T, sp); break;
+            case 3: as_rowB_body<3, true>(net, st, sc, L, li, valid, s, i, lane, T, sp); break;
+            case 4: as_rowB_body<4, true>(net, st, sc, L, li, valid, s, i, lane, T, sp); break;
+            case 5: as_rowB_body<5, true>(net, st, sc, L, li, valid, s, i, lane, T, sp); break;
+            case 6: as_rowB_body<6, true>(net, st, sc, L, li, valid, s, i, lane, T, sp); break;
+            case 7: as_rowB_body<7, true>(net, st, sc, L, li, valid, s, i, lane, T, sp); break;
+            default: as_rowB_body<8, true>(net, st, sc, L, li, valid, s, i, lane, T, sp); break;
         }
     } else {
         switch (ns) {
-            case 0: as_rowB_body<0, false>(net, st, sc, L, li, valid, s, i, lane, T, sp, it); break;
-            case 1: as_rowB_body<1, false>(net, st, sc, L, li, valid, s, i, lane, T, sp, it); break;
-            case 2: as_rowB_body<2, false>(net, st, sc, L, li, valid, s, i, lane, T, sp, it); break;
-            case 3: as_rowB_body<3, false>(net, st, sc, L, li, valid, s, i, lane, T, sp, it); break;
-            case 4: as_rowB_body<4, false>(net, st, sc, L, li, valid, s, i, lane, T, sp, it); break;
-            case 5: as_rowB_body<5, false>(net, st, sc, L, li, valid, s, i, lane, T, sp, it); break;
-            case 6: as_rowB_body<6, false>(net, st, sc, L, li, valid, s, i, lane, T, sp, it); break;
-            case 7: as_rowB_body<7, false>(net, st, sc, L, li, valid, s, i, lane, T, sp, it); break;
-            default: as_rowB_body<8, false>(net, st, sc, L, li, valid, s, i, lane, T, sp, it); break;
+            case 0: as_rowB_body<0, false>(net, st, sc, L, li, valid, s, i, lane, T, sp); break;
+            case 1: as_rowB_body<1, false>(net, st, sc, L, li, valid, s, i, lane, T, sp); break;
+            case 2: as_rowB_body<2, false>(net, st, sc, L, li, valid, s, i, lane, T, sp); break;
+            case 3: as_rowB_body<3, false>(net, st, sc, L, li, valid, s, i, lane, T, sp); break;
+            case 4: as_rowB_body<4, false>(net, st, sc, L, li, valid, s, i, lane, T, sp); break;
+            case 5: as_rowB_body<5, false>(net, st, sc, L, li, valid, s, i, lane, T, sp); break;
+            case 6: as_rowB_body<6, false>(net, st, sc, L, li, valid, s, i, lane, T, sp); break;
+            case 7: as_rowB_body<7, false>(net, st, sc, L, li, valid, s, i, lane, T, sp); break;
+            default: as_rowB_body<8, false>(net, st, sc, L, li, valid, s, i, lane, T, sp); break;
         }
     }
     if (staged) {
@@ -1225,7 +1005,7 @@ __global__ void __launch_bounds__(CB_THREADS, 4) k_slot_sums_t(DNet net, DState 
 // records, or with tc the BF16 form's bf16 operand planes.
 __global__ void k_rowprep(DNet net, DState st, DSched sc, int tc) {
     const size_t n = (size_t)net.S * net.NH;
-    const Step sp = cb_step(st.ctr[0], sc, st.lr_tab);
+    const StepNow sp = cb_step(st);
     const int bo = sp.nadd_before & 1;
     for (size_t u = blockIdx.x * (size_t)blockDim.x + threadIdx.x; u < n; u += (size_t)gridDim.x * blockDim.x) {
         const int s = (int)(u / net.NH), hh = (int)(u - (size_t)s * net.NH);
@@ -1587,7 +1367,7 @@ __global__ void __launch_bounds__(CB_THREADS) k_sp_convert_P_t(DNet net, DState 
     if (li >= net.n - 1) return;   // the output layer's inputs carry no P (whole block)
     const DLayer& L = net.L[li];
     const Unit u = team_unit(sg, q, L.n_in, net.S);
-    const Step sp = cb_step(st.ctr[0], sc, st.lr_tab);
+    const StepNow sp = cb_step(st);
     const int nsl = u.valid ? min(sp.nadd_before, st.caps[u.s]) : 0;
     const int bo = sp.nadd_before & 1;
     const size_t xo = (size_t)u.s * net.NT + L.in_off + u.idx;

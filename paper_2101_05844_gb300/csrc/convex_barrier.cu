@@ -1,6 +1,7 @@
 // Host side of the convex-barrier C ABI (include/convex_barrier.h): context creation, buffer
 // layout in device memory, the Big-M / Active Set and Saddle Point iteration loops (optionally
 // captured as CUDA graphs), bound evaluation and state access.
+#include <algorithm>
 #include <cmath>
 #include <cstdlib>
 #include <cstdarg>
@@ -13,6 +14,7 @@
 #include "cb_kernels.cuh"
 #include "cb_backward.cuh"
 #include "cb_team.cuh"
+#include "cb_tile.cuh"
 #include "cb_tc.cuh"
 
 using namespace cb;
@@ -38,6 +40,12 @@ struct as_ctx {
     int blocksA = 0, blocksB = 0;
     TSegs tA{}, tB{};                // lane-team launch geometry of the Active Set passes
     int blocksTA = 0, blocksTB = 0;
+    // layers whose float32 walks go by tiles (row and col pass), and the lane teams' share beside them
+    bool tl_row[CB_MAXL] = {}, tl_col[CB_MAXL] = {};
+    TlSegs tlA{}, tlB{};
+    int blocksLA = 0, blocksLB = 0, smemLA = 0, smemLB = 0;
+    TSegs tAr{}, tBr{};
+    int blocksTAr = 0, blocksTBr = 0;
     cudaGraphExec_t g_as = nullptr, g_sp = nullptr;
     int g_as_len = 0, g_sp_len = 0, g_as_nodes = 0, g_sp_nodes = 0;
     float* Wlast = nullptr;        // original last layer [n_out][n_{n-1}] and bias
@@ -302,6 +310,242 @@ struct Bump {
     }
 };
 
+// ------------------------------------------------------------------------- tiled walks
+// The tile shape (lane warps, and with them channels and window) of one segment: g holds the layer's
+// geometry (P, Wq, C, SC, kt), lines the rows of its position grid, span the window rows a line takes
+// beyond its step. Taken is the shape whose tiles cost least, counted in cycles of an SM per source
+// channel: 12 per tap and warp (six packed FMAs of a pair of sums at half rate, four channels, over
+// four schedulers), and the staged bytes at 32 a cycle. False: no shape fits the shared memory.
+static bool tile_shape(TlSeg& g, int S, bool linear, int lines, int span, int rb, int eb) {
+    double best = -1;
+    g.ch = g.C <= 4 ? 4 : 8;
+    TlSeg take = g;
+    for (int lw = 1; lw <= 8; lw *= 2) {
+        TlSeg t = g;
+        t.lw = lw;
+        const int LT = tl_lanes(t), TC = tl_channels(t);
+        t.nct = (t.C + TC - 1) / TC;
+        t.npt = 1;
+        if (linear) {
+            t.nsub = LT;
+            t.WX = t.WN = 1;
+            t.CS = LT + 1;   // odd: the copies of neighbouring source channels spread over the banks
+        } else {
+            int nl = lines;
+            t.nsub = std::max(1, LT / t.P);
+            if (t.nsub == 1) {
+                t.npt = (t.P + LT - 1) / LT;
+                nl = 0;
+                for (int p0 = 0; p0 < t.P; p0 += LT)
+                    nl = std::max(nl, std::min(p0 + LT, t.P) - 1 - (p0 - p0 % t.Wq));
+                nl = nl / t.Wq + 1;
+            }
+            t.WN = ((nl - 1) * t.step + span) * t.WX;
+            t.CS = t.nsub * t.WN;
+        }
+        t.CK = 1;
+        auto fits = [&](int ck) {
+            TlSeg q = t;
+            q.CK = ck;
+            return tl_records(q) * (2 * rb + eb) <= 48 * 1024 && ck * q.kt * TC * 8 <= 16 * 1024;
+        };
+        if (linear) {
+            while (2 * t.CK <= 64 && t.CK < t.SC && fits(2 * t.CK)) t.CK *= 2;
+        } else {
+            while (t.CK < t.SC && t.CK < 64 && fits(t.CK + 1)) ++t.CK;
+        }
+        if (tl_smem(t, rb, 8, eb, 0) > 100 * 1024) continue;
+        const double cost = (double)tl_tiles(t, S) * t.SC *
+                            (t.kt * 24.0 * t.ch + t.nsub * t.WN * (rb / 32.0) + t.kt * TC * 8 / 32.0);
+        if (best < 0 || cost < best) {
+            best = cost;
+            take = t;
+        }
+    }
+    if (best < 0) return false;
+    g = take;
+    g.nch = g.SC ? (g.SC + g.CK - 1) / g.CK : 0;
+    return true;
+}
+
+// The segments of the tiled passes: which layers take them, their shapes, splits, weights and offsets.
+static int build_tiles(as_ctx* c, const std::vector<std::vector<float>>& Wh) {
+    DNet& D = c->net;
+    const int n = D.n, S = D.S;
+    struct Plan {
+        TlSeg g;
+        std::vector<int> ofs;   // window offsets of a source channel's taps
+    };
+    std::vector<Plan> pa, pb;
+    const int rb_col = tl_arec_bytes(1 + D.cap), rb_row = 8, eb_row = 8 * D.cap;
+    // Below about 30 M multiply-adds a pass (and slot) lane teams are faster: tiles leave most of the GPU
+    // idle, and splitting them costs a round through memory. Measured on the Wide conv net (0.93 M per
+    // subproblem), an iteration of five slots: 9 subproblems (8 M) 52 us by teams, 95 by tiles; 30 (28 M)
+    // the same; 250 (232 M) 2.7 times faster by tiles.
+    double work = 0;
+    for (int k = 0; k + 1 < n; ++k) work += (double)S * D.L[k].ho * D.L[k].wo * (double)Wh[k].size();
+    if (work < 3e7) return AS_OK;
+    for (int k = 0; k + 1 < n; ++k) {
+        const DLayer& L = D.L[k];
+        size_t nnz = 0;
+        for (float w : Wh[k]) nnz += w != 0.f;
+        if (2 * nnz < Wh[k].size()) continue;   // sparse weights: the tap lists leave the zeros out
+        const bool lin = L.kind == 0;
+        {
+            Plan p{};
+            TlSeg& g = p.g;
+            g.li = k;
+            g.P = lin ? 1 : L.ho * L.wo;
+            g.Wq = lin ? 1 : L.wo;
+            g.C = L.co;
+            g.SC = L.ci;
+            g.kt = lin ? 1 : L.kh * L.kw;
+            g.step = lin ? 1 : L.st;
+            g.WX = L.Wp;
+            g.rows = L.Hp;
+            g.cs = lin ? 1 : L.Hp * L.Wp;
+            for (int y = 0; y < (lin ? 1 : L.kh); ++y)
+                for (int x = 0; x < (lin ? 1 : L.kw); ++x) p.ofs.push_back(y * L.Wp + x);
+            if (tile_shape(g, S, lin, lin ? 1 : L.ho, lin ? 1 : L.kh, rb_row, eb_row)) {
+                c->tl_row[k] = true;
+                pb.push_back(p);
+            }
+        }
+        // every stride phase of a conv has to have taps and the launch room for its phases
+        if (!lin && (L.st > std::min(L.kh, L.kw) || (int)pa.size() + L.st * L.st + n > TL_MAXSEG)) continue;
+        std::vector<Plan> ph;
+        bool ok = true;
+        for (int py = 0; py < (lin ? 1 : L.st) && ok; ++py)
+            for (int px = 0; px < (lin ? 1 : L.st) && ok; ++px) {
+                Plan p{};
+                TlSeg& g = p.g;
+                g.li = k;
+                g.C = L.ci;
+                g.SC = L.co;
+                g.step = 1;
+                g.P = g.Wq = g.kt = 1;
+                int ny = 1, nky = 1, nkx = 1;
+                if (!lin) {
+                    // inputs of the phase: (y + pad) % st == py, i.e. y = (y0 + Y) st + py - pad
+                    auto count = [&](int size, int ph_, int& first) {
+                        int cnt = 0;
+                        first = 0;
+                        for (int y = 0; y < size; ++y)
+                            if ((y + L.pd) % L.st == ph_) {
+                                if (!cnt) first = (y + L.pd) / L.st;
+                                ++cnt;
+                            }
+                        return cnt;
+                    };
+                    g.py = py;
+                    g.px = px;
+                    ny = count(L.hi, py, g.y0);
+                    const int nx = count(L.wi, px, g.x0);
+                    if (ny * nx == 0) continue;
+                    nky = (L.kh - py + L.st - 1) / L.st;
+                    nkx = (L.kw - px + L.st - 1) / L.st;
+                    g.P = ny * nx;
+                    g.Wq = nx;
+                    g.kt = nky * nkx;
+                    g.WX = L.Wpo;
+                    g.rows = L.Hpo;
+                    g.cs = L.Hpo * L.Wpo;
+                    g.row0 = g.y0 + L.hl - (nky - 1);
+                    g.base = (nky - 1) * L.Wpo + g.x0 + L.wl;
+                } else {
+                    g.rows = 1;
+                    g.cs = 1;
+                }
+                for (int dy = 0; dy < nky; ++dy)
+                    for (int dx = 0; dx < nkx; ++dx) p.ofs.push_back(lin ? 0 : -(dy * L.Wpo + dx));
+                ok = tile_shape(g, S, lin, ny, nky, rb_col, 0);
+                ph.push_back(p);
+            }
+        if (!ok) continue;
+        c->tl_col[k] = true;
+        pa.insert(pa.end(), ph.begin(), ph.end());
+    }
+    if (!pa.empty()) {   // the output layer's inputs take no product: they go with the tiled launch
+        c->tl_col[n - 1] = true;
+        Plan p{};
+        p.g.li = n - 1;
+        p.g.P = p.g.Wq = p.g.step = p.g.kt = p.g.CK = p.g.WX = p.g.WN = p.g.CS = 1;
+        p.g.C = D.L[n - 1].n_in;
+        p.g.ch = 4;
+        p.g.lw = 1;
+        p.g.nsub = 32;
+        p.g.npt = 1;
+        p.g.nct = (p.g.C + 31) / 32;
+        pa.push_back(p);
+    }
+    size_t part = 0;
+    int ctrs = 0;
+    auto finish = [&](std::vector<Plan>& plans, TlSegs& segs, int& blocks, int& smem, bool col) -> int {
+        const int nv = col ? 1 : 1 + D.cap, rb = col ? rb_col : rb_row, eb = col ? 0 : eb_row;
+        // a tile whose walk is long against an even share of the launch over the SMs (two blocks each) is
+        // split; at least 64 taps per split
+        double total = 0;
+        for (const Plan& p : plans) total += (double)tl_tiles(p.g, S) * p.g.SC * p.g.kt;
+        const double share = std::max(total / (152 * 2), 64.0);
+        for (Plan& p : plans) {
+            p.g.ks = 1;
+            const double taps = (double)p.g.SC * p.g.kt;
+            if (p.g.nch > 1 && taps > 1.5 * share)
+                p.g.ks = std::min({p.g.nch, 16, (int)std::ceil(taps / share)});
+        }
+        // the longest blocks first
+        std::stable_sort(plans.begin(), plans.end(), [](const Plan& a, const Plan& b) {
+            return (double)a.g.SC * a.g.kt / a.g.ks > (double)b.g.SC * b.g.kt / b.g.ks;
+        });
+        size_t used = 0;
+        for (Plan& p : plans) {
+            TlSeg& g = p.g;
+            const int tiles = tl_tiles(g, S);
+            g.first = blocks;
+            if (g.nch) {
+                std::vector<int> ofs(tl_offsets(g), 0);
+                for (int q = 0; q < g.CK; ++q)
+                    for (int t = 0; t < g.kt; ++t) ofs[q * g.kt + t] = q * g.CS + p.ofs[t];
+                const size_t cells = (size_t)g.SC * g.kt * g.nct * tl_channels(g);
+                int* dofs;
+                float* w;
+                float2* wpm;
+                TRY(dalloc(c, &dofs, ofs.size()));
+                TRY(dalloc(c, &w, cells));
+                TRY(dalloc(c, &wpm, cells));
+                CUDA_TRY(c, cudaMemcpy(dofs, ofs.data(), ofs.size() * sizeof(int), cudaMemcpyHostToDevice));
+                g.kofs = dofs;
+                tl_weights(D.L[g.li], col, g, w, wpm, c->stream);
+                CUDA_TRY(c, cudaGetLastError());
+                g.w = w;
+                g.wpm = wpm;
+                smem = std::max(smem, tl_smem(g, rb, 8, eb, nv));
+            }
+            if (g.ks > 1) {
+                g.part = used;
+                used += (size_t)tiles * g.ks * tl_split(g, nv);
+                g.ctr = ctrs;
+                ctrs += tiles;
+            }
+            blocks += tiles * g.ks;
+            segs.s[segs.n++] = g;
+        }
+        part = std::max(part, used);
+        return AS_OK;
+    };
+    TRY(finish(pa, c->tlA, c->blocksLA, c->smemLA, true));
+    TRY(finish(pb, c->tlB, c->blocksLB, c->smemLB, false));
+    if (ctrs) {
+        TRY(dalloc(c, &c->tlA.part, part));
+        TRY(dalloc(c, &c->tlA.ctr, (size_t)ctrs));
+        CUDA_TRY(c, cudaMemsetAsync(c->tlA.ctr, 0, (size_t)ctrs * sizeof(int), c->stream));
+        c->tlB.part = c->tlA.part;   // the passes of a context run one after the other
+        c->tlB.ctr = c->tlA.ctr;
+    }
+    CUDA_TRY(c, tl_as_prepare(c->smemLA, c->smemLB));
+    return AS_OK;
+}
+
 // Sign-partitioned tap lists and record layouts of the Active Set walks (DLayer fields) for the
 // hidden-output layers. Taps index record positions: the input records (one float2 each) for the
 // row pass, the output records (RS / 4 float4 planes) for the col pass.
@@ -467,6 +711,22 @@ static int make_team_segs(as_ctx* c) {
     };
     TRY(build(c->tA, c->blocksTA, true));
     TRY(build(c->tB, c->blocksTB, false));
+    // the lane teams' share of the float32 Active Set passes
+    auto rest = [&](const TSegs& all, const bool* tiled, TSegs& sg, int& blocks) {
+        sg = TSegs{};
+        blocks = 0;
+        for (int q = 0; q < all.n; ++q) {
+            if (tiled[all.layer[q]]) continue;
+            sg.layer[sg.n] = all.layer[q];
+            sg.T[sg.n] = all.T[q];
+            sg.perm[sg.n] = all.perm[q];
+            sg.start[sg.n++] = blocks;
+            blocks += all.start[q + 1] - all.start[q];
+        }
+        sg.start[sg.n] = blocks;
+    };
+    rest(c->tA, c->tl_col, c->tAr, c->blocksTAr);
+    rest(c->tB, c->tl_row, c->tBr, c->blocksTBr);
     return AS_OK;
 }
 
@@ -493,6 +753,7 @@ static int alloc_state(as_ctx* c) {
         }
         st.ctr = z.take<int>(4);
         st.status = z.take<int>(1);
+        st.step = z.take<Step>(1);
         Bump o{pass ? c->work_arena : nullptr, 0};
         st.lo = o.take<float>(NTS);
         st.hi = o.take<float>(NTS);
@@ -576,7 +837,7 @@ static int load_batch(as_ctx* c, const float* x_lo, const float* x_hi, const flo
     TRY(clear_planes(c));
     c->bounds_ibp = lhat == nullptr;
     c->have_splits = splits != nullptr && lhat == nullptr;
-    LAUNCH(c, s, CB_K_BATCH, (k_fill<<<grid_for(S), CB_THREADS, 0, s>>>(st.best, (size_t)S, -INFINITY)));
+    LAUNCH(c, s, CB_K_BATCH, (k_start<<<grid_for(S), CB_THREADS, 0, s>>>(st, c->sc, S)));
     c->sp_started = false;
     if (host_checks) {
         std::vector<float> hl((size_t)S * n0), hh((size_t)S * n0);
@@ -680,8 +941,10 @@ static int time_iters(as_ctx* c, int reps, float* ms) {
     const int it = c->sc.ntab - 2 > 0 ? c->sc.ntab - 2 : 0;
     int w[3] = {it, 0, 0};
     CUDA_TRY(c, cudaMemcpyAsync(c->st.ctr, w, sizeof w, cudaMemcpyHostToDevice, c->stream));
+    k_set_step<<<1, 32, 0, c->stream>>>(c->st, c->sc);
     TRY(launch_as_iter(c, c->stream));
     CUDA_TRY(c, cudaMemcpyAsync(c->st.ctr, w, sizeof w, cudaMemcpyHostToDevice, c->stream));
+    k_set_step<<<1, 32, 0, c->stream>>>(c->st, c->sc);
     cudaEvent_t a, b;
     CUDA_TRY(c, cudaEventCreate(&a));
     CUDA_TRY(c, cudaEventCreate(&b));
@@ -797,6 +1060,7 @@ static int init_impl(as_ctx* c, const as_net* net, int S, const float* x_lo, con
         }
     }
     TRY(build_walks(c, Wh));
+    TRY(build_tiles(c, Wh));
     // launch geometry
     {
         std::vector<int> ids;
@@ -869,15 +1133,29 @@ extern "C" void as_destroy(as_ctx* c) {
 }
 
 // ------------------------------------------------------------------------------- iterations
+// The float32 col pass: the tiled layers, then the lane teams' share. Mode 1 (the bound's evaluation
+// at the current duals) takes the sums in the lane teams' order.
+static void launch_colA(as_ctx* c, cudaStream_t s, int mode) {
+    if (c->blocksLA)
+        LAUNCH(c, s, CB_K_AS_COLA,
+               tl_launch_colA(mode == 1, c->blocksLA, c->smemLA, c->net, c->st, c->sc, c->tlA, mode, s));
+    if (c->blocksTAr)
+        LAUNCH(c, s, CB_K_AS_COLA,
+               (k_as_colA_t<false><<<c->blocksTAr, CB_THREADS, 0, s>>>(c->net, c->st, c->sc, c->tAr, mode)));
+}
+
 static int launch_as_iter(as_ctx* c, cudaStream_t s) {
     // the per-neuron bound terms are only summed when the best bound is tracked
     const int mode = c->opt.track_best ? 0 : 2;
-    LAUNCH(c, s, CB_K_AS_COLA, (k_as_colA_t<false><<<c->blocksTA, CB_THREADS, 0, s>>>(c->net, c->st, c->sc, c->tA, mode)));
+    launch_colA(c, s, mode);
     if (c->net.ball) LAUNCH(c, s, CB_K_BALL_X0, (k_ball_x0<<<c->net.S, CB_BALL_THREADS, 0, s>>>(c->net, c->st)));
     if (c->opt.track_best)
         LAUNCH(c, s, CB_K_REDUCE, (k_reduce<<<c->net.S, CB_THREADS, 0, s>>>(c->net, c->st, 64, nullptr, 1)));
-    LAUNCH(c, s, CB_K_AS_ROWB, (k_as_rowB_t<false><<<c->blocksTB, CB_THREADS, 0, s>>>(c->net, c->st, c->sc, c->tB)));
-    LAUNCH(c, s, CB_K_COUNTER, (k_advance<<<1, 1, 0, s>>>(c->st.ctr, 0)));
+    if (c->blocksLB)
+        LAUNCH(c, s, CB_K_AS_ROWB, tl_launch_rowB(c->blocksLB, c->smemLB, c->net, c->st, c->sc, c->tlB, s));
+    if (c->blocksTBr)
+        LAUNCH(c, s, CB_K_AS_ROWB, (k_as_rowB_t<false><<<c->blocksTBr, CB_THREADS, 0, s>>>(c->net, c->st, c->sc, c->tBr)));
+    LAUNCH(c, s, CB_K_COUNTER, (k_advance<<<1, 32, 0, s>>>(c->st, c->sc, 0)));
     return check_launch(c, "Active Set iteration");
 }
 
@@ -886,7 +1164,7 @@ static int launch_as_iter(as_ctx* c, cudaStream_t s) {
 static int launch_sp_iter(as_ctx* c, cudaStream_t s) {
     LAUNCH(c, s, CB_K_SP_ROWB, (k_sp_rowB_t<<<c->blocksTB, CB_THREADS, 0, s>>>(c->net, c->st, c->sc, c->tB)));
     LAUNCH(c, s, CB_K_SP_COLC, (k_sp_colCA_t<<<c->blocksTA, CB_THREADS, 0, s>>>(c->net, c->st, c->sc, c->tA)));
-    LAUNCH(c, s, CB_K_COUNTER, (k_advance<<<1, 1, 0, s>>>(c->st.ctr, 1)));
+    LAUNCH(c, s, CB_K_COUNTER, (k_advance<<<1, 32, 0, s>>>(c->st, c->sc, 1)));
     if (c->net.ball) LAUNCH(c, s, CB_K_BALL_X0, (k_ball_sp<<<c->net.S, CB_BALL_THREADS, 0, s>>>(c->net, c->st, 0)));
     if (c->opt.track_best)
         LAUNCH(c, s, CB_K_REDUCE, (k_reduce<<<c->net.S, CB_THREADS, 0, s>>>(c->net, c->st, 64, nullptr, 1)));
@@ -967,7 +1245,7 @@ static int sp_start(as_ctx* c) {
     for (int t = 0; t < c->opt.sp_init_steps; ++t) {
         LAUNCH(c, s, CB_K_SPI_ROW, (k_spi_row_t<<<c->blocksTB, CB_THREADS, 0, s>>>(c->net, c->st, c->tB)));
         LAUNCH(c, s, CB_K_SPI_COL, (k_spi_col_t<<<c->blocksTA, CB_THREADS, 0, s>>>(c->net, c->st, c->sc, c->tA)));
-        LAUNCH(c, s, CB_K_COUNTER, (k_advance<<<1, 1, 0, s>>>(c->st.ctr, 2)));
+        LAUNCH(c, s, CB_K_COUNTER, (k_advance<<<1, 32, 0, s>>>(c->st, c->sc, 2)));
         if (c->net.ball)
             LAUNCH(c, s, CB_K_BALL_X0, (k_ball_retract<<<c->net.S, CB_BALL_THREADS, 0, s>>>(c->net, c->st)));
     }
@@ -1003,7 +1281,7 @@ extern "C" int as_bound(as_ctx* c, int precision, double* out, double* best) {
     } else {
         // the BF16 form's iterates give a bound through float32 lambda, kappa and records
         if (c->opt.precision == 16) TRY(recompute_slot_sums(c));
-        LAUNCH(c, s, CB_K_AS_COLA, (k_as_colA_t<false><<<c->blocksTA, CB_THREADS, 0, s>>>(c->net, c->st, c->sc, c->tA, 1)));
+        launch_colA(c, s, 1);
         if (c->net.ball) LAUNCH(c, s, CB_K_BALL_X0, (k_ball_x0<<<S, CB_BALL_THREADS, 0, s>>>(c->net, c->st)));
     }
     double* dout = c->bound_out;
@@ -1180,6 +1458,7 @@ extern "C" int as_set_state(as_ctx* c, int which, const void* src) {
         if (v[0] < 0 || v[1] < 0) return fail(c, AS_ERR_ARG, "negative iteration counter");
         int w[3] = {v[0], v[1], v[2] ? c->opt.sp_init_steps : 0};
         CUDA_TRY(c, cudaMemcpyAsync(c->st.ctr, w, sizeof w, cudaMemcpyHostToDevice, c->stream));
+    k_set_step<<<1, 32, 0, c->stream>>>(c->st, c->sc);
         CUDA_TRY(c, cudaStreamSynchronize(c->stream));
         c->sp_started = v[2] != 0;
         return recompute_slot_sums(c);
