@@ -133,6 +133,7 @@ static int clear_planes(as_ctx* c);
 static int build_bf16(as_ctx* c, const std::vector<std::vector<float>>& Wh);
 static int autotune_tc(as_ctx* c);
 static int recompute_slot_sums(as_ctx* c);
+static int float_records(as_ctx* c);
 
 extern "C" void as_default_options(as_options* o) {
     if (!o) return;
@@ -1232,7 +1233,6 @@ extern "C" int as_step(as_ctx* c, int n_iters) {
 
 static int sp_start(as_ctx* c) {
     cudaStream_t s = c->stream;
-    if (c->opt.precision == 16) TRY(recompute_slot_sums(c));   // float32 lambda, kappa for the conversion
     const size_t NHS = (size_t)c->net.S * c->net.NH;
     LAUNCH(c, s, CB_K_SP_START, (k_sp_convert_elem<<<grid_for(NHS), CB_THREADS, 0, s>>>(c->net, c->st, c->sc,
                                                                                       (float)c->opt.sp_c_alpha,
@@ -1279,8 +1279,8 @@ extern "C" int as_bound(as_ctx* c, int precision, double* out, double* best) {
         LAUNCH(c, s, CB_K_SP_COLA, (k_sp_colA_t<<<c->blocksTA, CB_THREADS, 0, s>>>(c->net, c->st, c->tA, 0)));
         if (c->net.ball) LAUNCH(c, s, CB_K_BALL_X0, (k_ball_sp<<<S, CB_BALL_THREADS, 0, s>>>(c->net, c->st, 0)));
     } else {
-        // the BF16 form's iterates give a bound through float32 lambda, kappa and records
-        if (c->opt.precision == 16) TRY(recompute_slot_sums(c));
+        // the BF16 form's iterates give a bound through float32 records (its lambda, kappa are float32)
+        if (c->opt.precision == 16) TRY(float_records(c));
         launch_colA(c, s, 1);
         if (c->net.ball) LAUNCH(c, s, CB_K_BALL_X0, (k_ball_x0<<<S, CB_BALL_THREADS, 0, s>>>(c->net, c->st)));
     }
