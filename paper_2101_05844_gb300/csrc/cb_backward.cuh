@@ -55,7 +55,7 @@ __device__ __forceinline__ float wgrad_term(const DNet& net, const DState& st, c
     return g;
 }
 
-// Linear hidden layer: one thread per (i, j), summing over subproblems.
+// Linear hidden layer over an ellipsoid's layer 1: one thread per (i, j), summing over subproblems.
 __global__ void k_grad_W_linear(DNet net, DState st, int li, GradCtx gc, float* dW) {
     const DLayer& L = net.L[li];
     const size_t n = (size_t)L.n_out * L.n_in;
@@ -69,6 +69,92 @@ __global__ void k_grad_W_linear(DNet net, DState st, int li, GradCtx gc, float* 
         }
         dW[u] += (float)acc;
     }
+}
+
+// The same sums tile by tile (not for layer 1 over an ellipsoid): a block takes 32 rows x 64 columns, a
+// thread eight rows of one column, and a row's duals, snapshot bits and slots are staged for 16
+// subproblems at a time, where a thread per weight read them from L1 for itself alone. Every weight's
+// float64 sum runs over the subproblems in order, as above. 256 subproblems, 1024 x 1024, three slots:
+// 2885 us by a thread per weight; the float64 FMAs alone take about 420.
+constexpr int CB_GW_I = 32, CB_GW_J = 64, CB_GW_S = 16, CB_GW_R = CB_GW_I * CB_GW_J / CB_THREADS;
+template <int NS, bool CHAIN>
+__global__ void __launch_bounds__(CB_THREADS) k_grad_W_tile(DNet net, DState st, int li, GradCtx gc, float* dW) {
+    __shared__ float ab[CB_GW_S][CB_GW_I], bs[NS > 0 ? NS : 1][CB_GW_S][CB_GW_I];
+    __shared__ float ah[CHAIN ? CB_GW_S : 1][CB_GW_I], uh[CHAIN ? CB_GW_S : 1][CB_GW_I];
+    __shared__ unsigned zz[CB_GW_S][CB_GW_I];   // snapshot bits of z | z* << 8
+    __shared__ double gs[CB_GW_S];
+    const DLayer& L = net.L[li];
+    const int i0 = blockIdx.y * CB_GW_I, j = blockIdx.x * CB_GW_J + (threadIdx.x & (CB_GW_J - 1));
+    const int r0 = threadIdx.x / CB_GW_J * CB_GW_R;
+    const size_t NT = net.NT, NH = net.NH;
+    const bool on = j < L.n_in;
+    float w[CB_GW_R];
+    double acc[CB_GW_R];
+#pragma unroll
+    for (int r = 0; r < CB_GW_R; ++r) {
+        acc[r] = 0.0;
+        w[r] = on && i0 + r0 + r < L.n_out ? L.W[(size_t)(i0 + r0 + r) * L.n_in + j] : 0.f;
+    }
+    for (int s0 = 0; s0 < net.S; s0 += CB_GW_S) {
+        const int ns = min(CB_GW_S, net.S - s0);
+        __syncthreads();
+        for (int u = threadIdx.x; u < ns * CB_GW_I; u += CB_THREADS) {
+            const int q = u / CB_GW_I, r = u - q * CB_GW_I, s = s0 + q, i = i0 + r;
+            if (r == 0) gs[q] = gc.gb[s];
+            if (i >= L.n_out) continue;
+            const size_t h = (size_t)s * NH + L.h_out + i, hs = (size_t)s * net.cap * NH + L.h_out + i;
+            ab[q][r] = st.alpha[h] - st.beta1[h];
+            zz[q][r] = st.zsnap[gc.bo][h] | (st.zcur[h] ? 256u : 0u);
+            const int nsl = min(gc.nsl_before, st.caps[s]);
+#pragma unroll
+            for (int b = 0; b < NS; ++b) bs[b][q][r] = b < nsl ? st.bs[hs + (size_t)b * NH] : 0.f;
+            if constexpr (CHAIN) {
+                ah[q][r] = gc.Ah[h];
+                uh[q][r] = gc.Uh[h];
+            }
+        }
+        __syncthreads();
+        if (!on) continue;
+        for (int q = 0; q < ns; ++q) {
+            const size_t xo = (size_t)(s0 + q) * NT + L.in_off + j;
+            const float x = st.xval[xo];
+            float lo = 0.f, hi = 0.f;
+            unsigned pm = 0u, qm = 0u;
+            if (NS > 0 || CHAIN) {
+                lo = st.lo[xo];
+                hi = st.hi[xo];
+                slot_bits(net, L, st.xsnap[gc.bo][xo], lo == hi, pm, qm);
+            }
+            const double g = gs[q];
+#pragma unroll
+            for (int r = 0; r < CB_GW_R; ++r) {
+                float v = ab[q][r0 + r] * x;
+                const float Lc = w[r] >= 0.f ? lo : hi, Uc = w[r] >= 0.f ? hi : lo;
+                if constexpr (NS > 0) {
+                    const unsigned zb = zz[q][r0 + r];
+                    const unsigned I = zb | (w[r] > 0.f ? pm : w[r] < 0.f ? qm : 0xFFu);
+                    const float z = zb & 256u ? 1.f : 0.f;
+                    const float in = (1.f - z) * Lc - x, out = -z * Uc;
+#pragma unroll
+                    for (int b = 0; b < NS; ++b) v += bs[b][q][r0 + r] * ((I >> b) & 1u ? in : out);
+                }
+                if constexpr (CHAIN) v += ah[q][r0 + r] * Lc + uh[q][r0 + r] * Uc;
+                acc[r] += g * (double)v;
+            }
+        }
+    }
+    if (!on) return;
+#pragma unroll
+    for (int r = 0; r < CB_GW_R; ++r)
+        if (i0 + r0 + r < L.n_out) dW[(size_t)(i0 + r0 + r) * L.n_in + j] += (float)acc[r];
+}
+
+template <int NS>
+static void launch_grad_W_tile(const DNet& net, const DState& st, int li, const GradCtx& gc, float* dW, cudaStream_t s) {
+    const DLayer& L = net.L[li];
+    const dim3 grid((L.n_in + CB_GW_J - 1) / CB_GW_J, (L.n_out + CB_GW_I - 1) / CB_GW_I);
+    if (gc.Ah) k_grad_W_tile<NS, true><<<grid, CB_THREADS, 0, s>>>(net, st, li, gc, dW);
+    else k_grad_W_tile<NS, false><<<grid, CB_THREADS, 0, s>>>(net, st, li, gc, dW);
 }
 
 // Conv hidden layer: one block per filter entry, reducing over subproblems and positions.
