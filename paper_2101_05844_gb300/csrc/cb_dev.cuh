@@ -368,4 +368,158 @@ __device__ __forceinline__ void as_rowB_unit(const DNet& net, const DState& st, 
     put(0, contrib);
 }
 
+// ---------------------------------------------------------------- Saddle Point units
+// Saddle Point records, in the Active Set walks' layouts (Active Set and Saddle Point do not run on
+// one context at the same time, so the output records reuse the Active Set's array):
+//  per output position (the first float4 plane of the output records): {alpha, beta_bar on beta_1,
+//      beta_bar on I*, z} of the current iterate, written by the row pass (alpha also by k_sp_prep);
+//  per input position, two float4 planes (st.spin): {x, tau+, l, u} for W > 0 and {x, tau-, u, l}
+//      for W < 0, i.e. {x, threshold, Lcheck, Ucheck} for the sign of the taps that read it.
+__device__ __forceinline__ float4* sp_orec(const DNet& net, const DState& st, const DLayer& L, int s, int i) {
+    return arec_planes(net, st, L, s) + arec_pos(L, i);
+}
+// the W > 0 plane of layer L (the W < 0 plane follows, xpos float4 later): in float4 units a
+// layer takes 2 xpos, as it takes 2 xpos floats in the Active Set input records
+__device__ __forceinline__ float4* sp_iplane(const DNet& net, const DState& st, const DLayer& L, int s) {
+    return st.spin + (size_t)s * net.XT + (size_t)L.xo;
+}
+
+// Phase A epilogue for input j of layer L (k = li + 1, m = k - 1): f_m from acc = (W_k^T alpha_k)[j]
+// (Sec. 5.1), the primal conditional gradient (eqs. 7-8 with B = E), the bound terms, and the
+// records of input j for the row pass: the thresholds of the oracle eq. (3) at the primal iterate
+// x (buffer cur), rounded up to float32 (cb_tau_up) so that the row pass's compares are exact.
+// init != 0 also starts the primal iterate at the conditional gradient.
+__device__ __forceinline__ void sp_phaseA_epilogue(const DNet& net, const DState& st, const DLayer& L, int k,
+                                                   int s, int j, float acc, int cur, int init) {
+    const int m = k - 1;
+    const size_t NT = net.NT, NH = net.NH;
+    const size_t xo = (size_t)s * NT + L.in_off + j;
+    float f = k <= net.n - 1 ? st.P[xo] - acc : -net.Wout[(size_t)s * L.n_in + j];
+    const float lo = st.lo[xo], hi = st.hi[xo];
+    double term = 0.0;
+    if (m >= 1) {
+        const size_t h = (size_t)s * NH + L.h_in + j;
+        f += st.alpha[h] - st.Sb[h];
+        const float G = st.G[h];
+        const bool z = G >= 0.f;
+        st.zbar[h] = z;
+        if (init) st.spz[cur][h] = z ? 1.f : 0.f;
+        term = (double)net.L[m - 1].b[j] * st.alpha[h] + (double)st.C[h] - (z ? (double)G : 0.0);
+    }
+    const float xb = f >= 0.f ? hi : lo;
+    st.xbar[xo] = xb;
+    term -= (double)f * xb;
+    st.terms[xo] = term;
+    if (net.ball && L.in_off == 0) st.fval[xo] = f;   // for the ellipsoid vertex (k_ball_sp)
+    const float x = init ? xb : st.spx[cur][xo];
+    if (init) st.spx[cur][xo] = xb;
+    if (k <= net.n - 1) {
+        float tp = -INFINITY, tn = -INFINITY;
+        if (lo != hi) {
+            tp = cb_tau_up(x, lo, lo, hi);
+            tn = cb_tau_up(hi, x, lo, hi);
+        }
+        float4* r = sp_iplane(net, st, L, s) + xin_pos(L, j);
+        r[0] = make_float4(x, tp, lo, hi);
+        r[L.xpos] = make_float4(x, tn, hi, lo);
+    }
+}
+
+// Phase B of one row after its sums (a0 = W x, A = (W o I*) x, Lam, Mu the row sums of the oracle mask,
+// nout its unselected free inputs): conditional gradients alpha_bar (eq. 11) and beta_bar (eq. 12), the
+// convex combination of alpha, Sb, G, C at iteration t, and the output record.
+__device__ __forceinline__ void sp_rowB_unit(const DNet& net, const DState& st, const DSched& sc, const DLayer& L, int s,
+                                             int i, int t, float a0, float A, float Lam, float Mu, int nout) {
+    const int cur = t & 1;
+    const size_t NT = net.NT, h = (size_t)s * net.NH + L.h_out + i;
+    const float z = st.spz[cur][h];
+    // a row selecting none or all of its free inputs is the all-zero / all-ones constraint, a
+    // looser copy of beta_0 / beta_1: it does not compete in the choice of eq. (12)
+    const bool degenerate = nout == 0 || nout == st.nfree[h];
+    const float gamma = 1.f / ((float)t + sc.gamma0);
+    const float bi = L.b[i];
+    const float xhat = a0 + bi;
+    const float x = st.spx[cur][(size_t)s * NT + L.out_off + i];
+    const float uh = st.uhat[h], lh = st.lhat[h];
+    const float abar = (xhat - x >= 0.f) ? st.mua[h] : 0.f;
+    const float v0 = x - z * uh;
+    const float v1 = x - xhat + (1.f - z) * lh;
+    const float vI = x - A + (1.f - z) * Lam - z * (bi + Mu);
+    int sel = 0;
+    float vm = v0;
+    if (v1 > vm) { sel = 1; vm = v1; }
+    if (!degenerate && vI > vm) { sel = 2; vm = vI; }
+    const bool on = vm >= 0.f;
+    const float bb = on ? st.mub[h] : 0.f;
+    const float gsel = sel == 0 ? uh : (sel == 1 ? lh : Lam + Mu + bi);
+    const float csel = sel == 0 ? 0.f : (sel == 1 ? lh - bi : Lam);
+    const float om = 1.f - gamma;
+    const float an = om * st.alpha[h] + gamma * abar;
+    st.alpha[h] = an;
+    st.Sb[h] = om * st.Sb[h] + gamma * bb;
+    st.G[h] = om * st.G[h] + gamma * (bb * gsel);
+    st.C[h] = om * st.C[h] + gamma * (bb * csel);
+    st.sel[h] = on ? (uint8_t)sel : (uint8_t)3;
+    *sp_orec(net, st, L, s, i) = make_float4(an, sel == 1 ? bb : 0.f, sel == 2 ? bb : 0.f, z);
+}
+
+// Phase C of one input after its sums at iteration t, fused with phase A of the next (k_sp_colCA_t): the
+// convex combination of P_k (accC the masked backward product of the chosen masks) and of the primal
+// iterate into the other buffer, then phase A there (accA = (W^T alpha)[j]).
+__device__ __forceinline__ void sp_colC_unit(const DNet& net, const DState& st, const DSched& sc, const DLayer& L, int k,
+                                             int s, int j, int t, float accC, float accA) {
+    const int cur = t & 1, nxt = cur ^ 1;
+    const float gamma = 1.f / ((float)t + sc.gamma0);
+    const float om = 1.f - gamma;
+    const size_t xo = (size_t)s * net.NT + L.in_off + j;
+    if (k <= net.n - 1) st.P[xo] = om * st.P[xo] + gamma * accC;
+    st.spx[nxt][xo] = om * st.spx[cur][xo] + gamma * st.xbar[xo];
+    if (k >= 2) {
+        const size_t hh = (size_t)s * net.NH + L.h_in + j;
+        st.spz[nxt][hh] = om * st.spz[cur][hh] + gamma * (st.zbar[hh] ? 1.f : 0.f);
+    }
+    sp_phaseA_epilogue(net, st, L, k, s, j, accA, nxt, 0);
+}
+
+// Primal initialisation (App. C.2), one row after its sum a0 = W x: the inner maximisers at (x, z); returns
+// alpha* - beta_1*, the row's entry of the col pass.
+__device__ __forceinline__ float spi_row_unit(const DNet& net, const DState& st, const DLayer& L, int s, int i, int cur,
+                                              float a0) {
+    const size_t h = (size_t)s * net.NH + L.h_out + i;
+    const float xhat = a0 + L.b[i];
+    const float x = st.spx[cur][(size_t)s * net.NT + L.out_off + i];
+    const float z = st.spz[cur][h];
+    const float ab = (xhat - x >= 0.f) ? st.mua[h] : 0.f;
+    const float v0 = x - z * st.uhat[h];
+    const float v1 = x - xhat + (1.f - z) * st.lhat[h];
+    const bool on = fmaxf(v0, v1) >= 0.f;
+    const bool p0 = v0 >= v1;
+    const float b0 = (on && p0) ? st.mub[h] : 0.f;
+    const float b1 = (on && !p0) ? st.mub[h] : 0.f;
+    st.ab[h] = ab;
+    st.b0i[h] = b0;
+    st.b1i[h] = b1;
+    return ab - b1;
+}
+
+// Primal initialisation, one input after its sum acc = (W^T (alpha* - beta_1*))[j]: one step of x_m and z_m,
+// projected on the boxes (over an ellipsoid, k_ball_retract brings x_0 back into it); returns the new x.
+__device__ __forceinline__ float spi_col_unit(const DNet& net, const DState& st, const DSched& sc, const DLayer& L, int k,
+                                              int s, int j, int step, float acc) {
+    const int cur = st.ctr[1] & 1;
+    const float eta = sc.sp_lr0 + (sc.sp_lr1 - sc.sp_lr0) * (float)step / (float)max(1, sc.sp_init_steps - 1);
+    float f = k <= net.n - 1 ? -acc : -net.Wout[(size_t)s * L.n_in + j];
+    const size_t xo = (size_t)s * net.NT + L.in_off + j;
+    if (k >= 2) {
+        const size_t h = (size_t)s * net.NH + L.h_in + j;
+        f += st.ab[h] - st.b0i[h] - st.b1i[h];
+        const float g = st.b0i[h] * st.uhat[h] + st.b1i[h] * st.lhat[h];
+        st.spz[cur][h] = fminf(fmaxf(st.spz[cur][h] + eta * g, 0.f), 1.f);
+    }
+    float x = st.spx[cur][xo] + eta * f;
+    if (!(net.ball && L.in_off == 0)) x = fminf(fmaxf(x, st.lo[xo]), st.hi[xo]);
+    st.spx[cur][xo] = x;
+    return x;
+}
+
 }  // namespace cb

@@ -1002,7 +1002,8 @@ __global__ void __launch_bounds__(CB_THREADS, 4) k_slot_sums_t(DNet net, DState 
 }
 
 // rp and bz from the current duals and snapshots (after a state import): the float32 output
-// records, or with tc the BF16 form's bf16 operand planes.
+// records, or with tc = 1 the BF16 form's bf16 operand planes. tc = 2: the float32 records with beta_1 +
+// sum_b z_b beta_b for rp (no alpha), whose col pass is Saddle Point's P (eq. 10).
 __global__ void k_rowprep(DNet net, DState st, DSched sc, int tc) {
     const size_t n = (size_t)net.S * net.NH;
     const StepNow sp = cb_step(st);
@@ -1017,7 +1018,7 @@ __global__ void k_rowprep(DNet net, DState st, DSched sc, int tc) {
         const int i = hh - L.h_out;
         const int ap = arec_pos(L, i);
         long long roff = 0;
-        if (tc) {
+        if (tc == 1) {
             int co = i, oy = 0, ox = 0;
             if (L.kind == 1) {
                 const int hw = L.ho * L.wo;
@@ -1028,14 +1029,14 @@ __global__ void k_rowprep(DNet net, DState st, DSched sc, int tc) {
             roff = ((long long)(oy + L.hl) * L.Wpo + (ox + L.wl)) * net.bf[li].Cop + co;
         }
         auto put = [&](int e, float v) {
-            if (tc)
+            if (tc == 1)
                 reinterpret_cast<__nv_bfloat16*>(net.bf[li].R)[((long long)e * net.S + s) * net.bf[li].PR + roff] =
                     __float2bfloat16_rn(v);
             else
                 *arec_entry(net, st, L, s, ap, e) = v;
         };
-        float r = -(st.alpha[u] - st.beta1[u]);
-        for (int b = 0; b < (tc ? net.cap : net.RS - 1); ++b) {
+        float r = tc == 2 ? st.beta1[u] : -(st.alpha[u] - st.beta1[u]);
+        for (int b = 0; b < (tc == 1 ? net.cap : net.RS - 1); ++b) {
             float bv = 0.f;
             bool zb = false;
             if (b < net.cap) {
@@ -1112,21 +1113,6 @@ __device__ __forceinline__ Unit team_unit(const TSegs& sg, int q, int count, int
     return u;
 }
 
-// Saddle Point records, in the Active Set walks' layouts (Active Set and Saddle Point do not run on
-// one context at the same time, so the output records reuse the Active Set's array):
-//  per output position (the first float4 plane of the output records): {alpha, beta_bar on beta_1,
-//      beta_bar on I*, z} of the current iterate, written by the row pass (alpha also by k_sp_prep);
-//  per input position, two float4 planes (st.spin): {x, tau+, l, u} for W > 0 and {x, tau-, u, l}
-//      for W < 0, i.e. {x, threshold, Lcheck, Ucheck} for the sign of the taps that read it.
-__device__ __forceinline__ float4* sp_orec(const DNet& net, const DState& st, const DLayer& L, int s, int i) {
-    return arec_planes(net, st, L, s) + arec_pos(L, i);
-}
-// the W > 0 plane of layer L (the W < 0 plane follows, xpos float4 later): in float4 units a
-// layer takes 2 xpos, as it takes 2 xpos floats in the Active Set input records
-__device__ __forceinline__ float4* sp_iplane(const DNet& net, const DState& st, const DLayer& L, int s) {
-    return st.spin + (size_t)s * net.XT + (size_t)L.xo;
-}
-
 // alpha into the output records (Saddle Point start, state import).
 __global__ void k_sp_prep(DNet net, DState st) {
     const size_t n = (size_t)net.S * net.NH;
@@ -1135,47 +1121,6 @@ __global__ void k_sp_prep(DNet net, DState st) {
         int li = 0;
         while (li + 2 < net.n && hh >= net.L[li + 1].h_out) ++li;
         *sp_orec(net, st, net.L[li], s, hh - net.L[li].h_out) = make_float4(st.alpha[u], 0.f, 0.f, 0.f);
-    }
-}
-
-// Phase A epilogue for input j of layer L (k = li + 1, m = k - 1): f_m from acc = (W_k^T alpha_k)[j]
-// (Sec. 5.1), the primal conditional gradient (eqs. 7-8 with B = E), the bound terms, and the
-// records of input j for the row pass: the thresholds of the oracle eq. (3) at the primal iterate
-// x (buffer cur), rounded up to float32 (cb_tau_up) so that the row pass's compares are exact.
-// init != 0 also starts the primal iterate at the conditional gradient.
-__device__ __forceinline__ void sp_phaseA_epilogue(const DNet& net, const DState& st, const DLayer& L, int k,
-                                                   int s, int j, float acc, int cur, int init) {
-    const int m = k - 1;
-    const size_t NT = net.NT, NH = net.NH;
-    const size_t xo = (size_t)s * NT + L.in_off + j;
-    float f = k <= net.n - 1 ? st.P[xo] - acc : -net.Wout[(size_t)s * L.n_in + j];
-    const float lo = st.lo[xo], hi = st.hi[xo];
-    double term = 0.0;
-    if (m >= 1) {
-        const size_t h = (size_t)s * NH + L.h_in + j;
-        f += st.alpha[h] - st.Sb[h];
-        const float G = st.G[h];
-        const bool z = G >= 0.f;
-        st.zbar[h] = z;
-        if (init) st.spz[cur][h] = z ? 1.f : 0.f;
-        term = (double)net.L[m - 1].b[j] * st.alpha[h] + (double)st.C[h] - (z ? (double)G : 0.0);
-    }
-    const float xb = f >= 0.f ? hi : lo;
-    st.xbar[xo] = xb;
-    term -= (double)f * xb;
-    st.terms[xo] = term;
-    if (net.ball && L.in_off == 0) st.fval[xo] = f;   // for the ellipsoid vertex (k_ball_sp)
-    const float x = init ? xb : st.spx[cur][xo];
-    if (init) st.spx[cur][xo] = xb;
-    if (k <= net.n - 1) {
-        float tp = -INFINITY, tn = -INFINITY;
-        if (lo != hi) {
-            tp = cb_tau_up(x, lo, lo, hi);
-            tn = cb_tau_up(hi, x, lo, hi);
-        }
-        float4* r = sp_iplane(net, st, L, s) + xin_pos(L, j);
-        r[0] = make_float4(x, tp, lo, hi);
-        r[L.xpos] = make_float4(x, tn, hi, lo);
     }
 }
 
@@ -1221,7 +1166,7 @@ __global__ void __launch_bounds__(CB_THREADS) k_sp_rowB_t(DNet net, DState st, D
     const int s = u.s, i = u.idx;
     const int t = st.ctr[1];
     const int cur = t & 1;
-    const size_t NT = net.NT, NH = net.NH;
+    const size_t NH = net.NH;
     const size_t h = (size_t)s * NH + L.h_out + i;
     const float z = u.valid ? st.spz[cur][h] : 0.f;
     float a0 = 0.f, A = 0.f, Lam = 0.f, Mu = 0.f;
@@ -1267,34 +1212,7 @@ __global__ void __launch_bounds__(CB_THREADS) k_sp_rowB_t(DNet net, DState st, D
         for (int o = u.T >> 1; o > 0; o >>= 1) nout += __shfl_xor_sync(0xffffffffu, nout, o);
     }
     if (!u.valid || u.lane != 0) return;
-    // a row selecting none or all of its free inputs is the all-zero / all-ones constraint, a
-    // looser copy of beta_0 / beta_1: it does not compete in the choice of eq. (12)
-    const bool degenerate = nout == 0 || nout == st.nfree[h];
-    const float gamma = 1.f / ((float)t + sc.gamma0);
-    const float bi = L.b[i];
-    const float xhat = a0 + bi;
-    const float x = st.spx[cur][(size_t)s * NT + L.out_off + i];
-    const float uh = st.uhat[h], lh = st.lhat[h];
-    const float abar = (xhat - x >= 0.f) ? st.mua[h] : 0.f;
-    const float v0 = x - z * uh;
-    const float v1 = x - xhat + (1.f - z) * lh;
-    const float vI = x - A + (1.f - z) * Lam - z * (bi + Mu);
-    int sel = 0;
-    float vm = v0;
-    if (v1 > vm) { sel = 1; vm = v1; }
-    if (!degenerate && vI > vm) { sel = 2; vm = vI; }
-    const bool on = vm >= 0.f;
-    const float bb = on ? st.mub[h] : 0.f;
-    const float gsel = sel == 0 ? uh : (sel == 1 ? lh : Lam + Mu + bi);
-    const float csel = sel == 0 ? 0.f : (sel == 1 ? lh - bi : Lam);
-    const float om = 1.f - gamma;
-    const float an = om * st.alpha[h] + gamma * abar;
-    st.alpha[h] = an;
-    st.Sb[h] = om * st.Sb[h] + gamma * bb;
-    st.G[h] = om * st.G[h] + gamma * (bb * gsel);
-    st.C[h] = om * st.C[h] + gamma * (bb * csel);
-    st.sel[h] = on ? (uint8_t)sel : (uint8_t)3;
-    *sp_orec(net, st, L, s, i) = make_float4(an, sel == 1 ? bb : 0.f, sel == 2 ? bb : 0.f, z);
+    sp_rowB_unit(net, st, sc, L, s, i, t, a0, A, Lam, Mu, nout);
 }
 
 // Phase C of iteration t fused with phase A of iteration t + 1 (col pass over k = 1..n): one walk
@@ -1307,11 +1225,9 @@ __global__ void __launch_bounds__(CB_THREADS) k_sp_colCA_t(DNet net, DState st, 
     const int q = tseg_of(sg, blockIdx.x);
     const int li = sg.layer[q];
     const DLayer& L = net.L[li];
-    const int k = li + 1, m = k - 1;
+    const int k = li + 1;
     const Unit u = team_unit(sg, q, L.n_in, net.S);
     const int t = st.ctr[1];
-    const size_t NT = net.NT, NH = net.NH;
-    const size_t xo = (size_t)u.s * NT + L.in_off + u.idx;
     float accC = 0.f, accA = 0.f;
     if (u.valid && k <= net.n - 1) {
         const float4* own = sp_iplane(net, st, L, u.s) + xin_pos(L, u.idx);
@@ -1344,16 +1260,7 @@ __global__ void __launch_bounds__(CB_THREADS) k_sp_colCA_t(DNet net, DState st, 
         accA = team_sum(accA, u.T);
     }
     if (u.valid && u.lane == 0) {
-        const int cur = t & 1, nxt = cur ^ 1;
-        const float gamma = 1.f / ((float)t + sc.gamma0);
-        const float om = 1.f - gamma;
-        if (k <= net.n - 1) st.P[xo] = om * st.P[xo] + gamma * accC;
-        st.spx[nxt][xo] = om * st.spx[cur][xo] + gamma * st.xbar[xo];
-        if (m >= 1) {
-            const size_t hh = (size_t)u.s * NH + L.h_in + u.idx;
-            st.spz[nxt][hh] = om * st.spz[cur][hh] + gamma * (st.zbar[hh] ? 1.f : 0.f);
-        }
-        sp_phaseA_epilogue(net, st, L, k, u.s, u.idx, accA, nxt, 0);
+        sp_colC_unit(net, st, sc, L, k, u.s, u.idx, t, accC, accA);
     }
 }
 
@@ -1409,20 +1316,7 @@ __global__ void __launch_bounds__(CB_THREADS) k_spi_row_t(DNet net, DState st, T
     if (u.T > 1) a0 = team_sum(a0, u.T);
     if (!u.valid || u.lane != 0) return;
     const size_t h = (size_t)u.s * NH + L.h_out + u.idx;
-    const float xhat = a0 + L.b[u.idx];
-    const float x = st.spx[cur][(size_t)u.s * NT + L.out_off + u.idx];
-    const float z = st.spz[cur][h];
-    const float ab = (xhat - x >= 0.f) ? st.mua[h] : 0.f;
-    const float v0 = x - z * st.uhat[h];
-    const float v1 = x - xhat + (1.f - z) * st.lhat[h];
-    const bool on = fmaxf(v0, v1) >= 0.f;
-    const bool p0 = v0 >= v1;
-    const float b0 = (on && p0) ? st.mub[h] : 0.f;
-    const float b1 = (on && !p0) ? st.mub[h] : 0.f;
-    st.ab[h] = ab;
-    st.b0i[h] = b0;
-    st.b1i[h] = b1;
-    st.arow[h] = ab - b1;
+    st.arow[h] = spi_row_unit(net, st, L, u.s, u.idx, cur, a0);
 }
 
 // Primal initialisation, col pass: x_m += eta f_m(alpha*, beta*), z_m += eta g_m(beta*),
@@ -1431,10 +1325,10 @@ __global__ void __launch_bounds__(CB_THREADS) k_spi_col_t(DNet net, DState st, D
     const int q = tseg_of(sg, blockIdx.x);
     const int li = sg.layer[q];
     const DLayer& L = net.L[li];
-    const int k = li + 1, m = k - 1;
+    const int k = li + 1;
     const Unit u = team_unit(sg, q, L.n_in, net.S);
     const int step = st.ctr[2];
-    const size_t NT = net.NT, NH = net.NH;
+    const size_t NH = net.NH;
     float acc = 0.f;
     if (u.valid && k <= net.n - 1) {
         const float* ar = st.arow + (size_t)u.s * NH + L.h_out;
@@ -1442,20 +1336,7 @@ __global__ void __launch_bounds__(CB_THREADS) k_spi_col_t(DNet net, DState st, D
     }
     if (u.T > 1) acc = team_sum(acc, u.T);
     if (u.valid && u.lane == 0) {
-        const int cur = st.ctr[1] & 1;
-        const float eta = sc.sp_lr0 + (sc.sp_lr1 - sc.sp_lr0) * (float)step / (float)max(1, sc.sp_init_steps - 1);
-        float f = k <= net.n - 1 ? -acc : -net.Wout[(size_t)u.s * L.n_in + u.idx];
-        const size_t xo = (size_t)u.s * NT + L.in_off + u.idx;
-        if (m >= 1) {
-            const size_t h = (size_t)u.s * NH + L.h_in + u.idx;
-            f += st.ab[h] - st.b0i[h] - st.b1i[h];
-            const float g = st.b0i[h] * st.uhat[h] + st.b1i[h] * st.lhat[h];
-            st.spz[cur][h] = fminf(fmaxf(st.spz[cur][h] + eta * g, 0.f), 1.f);
-        }
-        if (net.ball && L.in_off == 0)   // over an ellipsoid, k_ball_retract brings x_0 back into it
-            st.spx[cur][xo] = st.spx[cur][xo] + eta * f;
-        else
-            st.spx[cur][xo] = fminf(fmaxf(st.spx[cur][xo] + eta * f, st.lo[xo]), st.hi[xo]);
+        spi_col_unit(net, st, sc, L, k, u.s, u.idx, step, acc);
     }
 }
 
@@ -1546,6 +1427,7 @@ __global__ void __launch_bounds__(CB_BALL_THREADS) k_ball_retract(DNet net, DSta
     for (int j = threadIdx.x; j < L.n_in; j += CB_BALL_THREADS) {
         const float lo = st.lo[base + j], hi = st.hi[base + j], c = 0.5f * (lo + hi);
         x[j] = lo != hi ? fminf(fmaxf(c + (x[j] - c) * scale, lo), hi) : c;
+        sp_iplane(net, st, L, s)[xin_pos(L, j)].x = x[j];   // the tiled row pass reads the records
     }
 }
 

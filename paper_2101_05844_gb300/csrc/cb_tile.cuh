@@ -297,6 +297,22 @@ void tl_launch_colA(bool seq, int blocks, int smem, const DNet& net, const DStat
                     int mode, cudaStream_t s);
 void tl_launch_rowB(int blocks, int smem, const DNet& net, const DState& st, const DSched& sc, const TlSegs& t,
                     cudaStream_t s);
+// Interval propagation (tile_sp.cu): the input box's records, then a row segment per hidden layer.
+int tl_ibp_smem(const TlSeg& g);
+cudaError_t tl_sp_prepare(int smem_ibp, int smem_row, int smem_col);
+void tl_launch_ibp_box(int grid, const DNet& net, const DState& st, cudaStream_t s);
+void tl_launch_ibp(const DNet& net, const DState& st, const TlSeg& seg, const signed char* splits, cudaStream_t s);
+// Saddle Point (tile_sp.cu): its passes, the col pass's work by `what` (0: phase C and the next phase A, 1:
+// phase A, 2: phase A starting the primal iterate, 3: a step of the primal initialisation).
+int tl_sp_row_smem(const TlSeg& g);
+int tl_sp_col_smem(const TlSeg& g);
+void tl_launch_sp_row(int blocks, int smem, const DNet& net, const DState& st, const DSched& sc, const TlSegs& t,
+                      cudaStream_t s);
+void tl_launch_sp_col(int what, int blocks, int smem, const DNet& net, const DState& st, const DSched& sc, const TlSegs& t,
+                      cudaStream_t s);
+void tl_launch_spi_row(int blocks, int smem, const DNet& net, const DState& st, const TlSegs& t, cudaStream_t s);
+void tl_launch_sp_convert(int blocks, int smem, const DNet& net, const DState& st, const DSched& sc, const TlSegs& t,
+                          cudaStream_t s);
 // record bytes of the Active Set passes with up to cap slots (pieces of 4, 8 or 16 bytes)
 __host__ __device__ constexpr int tl_piece(int entries) { return entries >= 3 ? 16 : 4 * entries; }
 __host__ __device__ constexpr int tl_arec_bytes(int entries) {

@@ -42,6 +42,9 @@ struct as_ctx {
     int blocksTA = 0, blocksTB = 0;
     // layers whose float32 walks go by tiles (row and col pass), and the lane teams' share beside them
     bool tl_row[CB_MAXL] = {}, tl_col[CB_MAXL] = {};
+    bool ibp_tiles = false;          // interval propagation by tiles (every row pass is)
+    bool sp_tiles = false;           // Saddle Point by tiles (every row and col pass is)
+    int smemSA = 0, smemSB = 0;
     TlSegs tlA{}, tlB{};
     int blocksLA = 0, blocksLB = 0, smemLA = 0, smemLB = 0;
     TSegs tAr{}, tBr{};
@@ -378,7 +381,8 @@ static int build_tiles(as_ctx* c, const std::vector<std::vector<float>>& Wh) {
         std::vector<int> ofs;   // window offsets of a source channel's taps
     };
     std::vector<Plan> pa, pb;
-    const int rb_col = tl_arec_bytes(1 + D.cap), rb_row = 8, eb_row = 8 * D.cap;
+    // (Saddle Point stages 16 and 20 bytes a record on the same tiles)
+    const int rb_col = std::max(16, tl_arec_bytes(1 + D.cap)), rb_row = 8, eb_row = std::max(24, 8 * D.cap);
     // Below about 30 M multiply-adds a pass (and slot) lane teams are faster: tiles leave most of the GPU
     // idle, and splitting them costs a round through memory. Measured on the Wide conv net (0.93 M per
     // subproblem), an iteration of five slots: 9 subproblems (8 M) 52 us by teams, 95 by tiles; 30 (28 M)
@@ -524,7 +528,7 @@ static int build_tiles(as_ctx* c, const std::vector<std::vector<float>>& Wh) {
             }
             if (g.ks > 1) {
                 g.part = used;
-                used += (size_t)tiles * g.ks * tl_split(g, nv);
+                used += (size_t)tiles * g.ks * tl_split(g, std::max(nv, col ? 2 : 5));
                 g.ctr = ctrs;
                 ctrs += tiles;
             }
@@ -534,6 +538,7 @@ static int build_tiles(as_ctx* c, const std::vector<std::vector<float>>& Wh) {
         part = std::max(part, used);
         return AS_OK;
     };
+    // (scratch and shared memory also serve Saddle Point's passes on the same tiles: 2 and 5 values per unit)
     TRY(finish(pa, c->tlA, c->blocksLA, c->smemLA, true));
     TRY(finish(pb, c->tlB, c->blocksLB, c->smemLB, false));
     if (ctrs) {
@@ -544,6 +549,13 @@ static int build_tiles(as_ctx* c, const std::vector<std::vector<float>>& Wh) {
         c->tlB.ctr = c->tlA.ctr;
     }
     CUDA_TRY(c, tl_as_prepare(c->smemLA, c->smemLB));
+    c->ibp_tiles = c->tlB.n == n - 1;
+    int ibp = 0;
+    for (int q = 0; q < c->tlB.n; ++q) ibp = std::max(ibp, tl_ibp_smem(c->tlB.s[q]));
+    c->sp_tiles = c->ibp_tiles && (int)std::count(c->tl_col, c->tl_col + n, true) == n;
+    for (int q = 0; q < c->tlB.n; ++q) c->smemSB = std::max(c->smemSB, tl_sp_row_smem(c->tlB.s[q]));
+    for (int q = 0; q < c->tlA.n; ++q) c->smemSA = std::max(c->smemSA, tl_sp_col_smem(c->tlA.s[q]));
+    CUDA_TRY(c, tl_sp_prepare(ibp, c->smemSB, c->smemSA));
     return AS_OK;
 }
 
@@ -892,8 +904,18 @@ static int load_batch(as_ctx* c, const float* x_lo, const float* x_hi, const flo
             CUDA_TRY(c, cudaMemcpyAsync(c->splits_dev, splits, NHS, cudaMemcpyDefault, s));
             dsp = c->splits_dev;
         }
+        // on tiles where the passes are (all layers have to be), except layer 1 over an ellipsoid
+        const bool tiled = c->ibp_tiles;
+        if (tiled && !D.ball)
+            LAUNCH(c, s, CB_K_BATCH, tl_launch_ibp_box(grid_for((size_t)S * n0), D, st, s));
         for (int k = 0; k < n - 1; ++k) {
             const long long warps = (long long)S * D.L[k].n_out;
+            if (tiled && !D.ball) {
+                for (int q = 0; q < c->tlB.n; ++q)
+                    if (c->tlB.s[q].li == k) LAUNCH(c, s, CB_K_BATCH, tl_launch_ibp(D, st, c->tlB.s[q], dsp, s));
+                TRY(check_launch(c, "k_ibp_tl"));
+                continue;
+            }
             LAUNCH(c, s, CB_K_BATCH, (k_ibp<<<(int)((warps + CB_WARPS - 1) / CB_WARPS), CB_THREADS, 0, s>>>(D, st, k, dsp)));
             TRY(check_launch(c, "k_ibp"));
         }
@@ -1160,11 +1182,24 @@ static int launch_as_iter(as_ctx* c, cudaStream_t s) {
     return check_launch(c, "Active Set iteration");
 }
 
+// Saddle Point's phase A alone; start: the primal iterate starts at its conditional gradient.
+static void launch_sp_phaseA(as_ctx* c, cudaStream_t s, int id, bool start) {
+    if (c->sp_tiles)
+        LAUNCH(c, s, id, tl_launch_sp_col(start ? 2 : 1, c->blocksLA, c->smemSA, c->net, c->st, c->sc, c->tlA, s));
+    else
+        LAUNCH(c, s, id, (k_sp_colA_t<<<c->blocksTA, CB_THREADS, 0, s>>>(c->net, c->st, c->tA, start ? 1 : 0)));
+}
+
 // One Saddle Point iteration t: phase B, then phase C fused with phase A of iteration t + 1 (the
 // loop's first phase A runs before it, k_sp_colA_t, whenever the state is new).
 static int launch_sp_iter(as_ctx* c, cudaStream_t s) {
-    LAUNCH(c, s, CB_K_SP_ROWB, (k_sp_rowB_t<<<c->blocksTB, CB_THREADS, 0, s>>>(c->net, c->st, c->sc, c->tB)));
-    LAUNCH(c, s, CB_K_SP_COLC, (k_sp_colCA_t<<<c->blocksTA, CB_THREADS, 0, s>>>(c->net, c->st, c->sc, c->tA)));
+    if (c->sp_tiles) {
+        LAUNCH(c, s, CB_K_SP_ROWB, tl_launch_sp_row(c->blocksLB, c->smemSB, c->net, c->st, c->sc, c->tlB, s));
+        LAUNCH(c, s, CB_K_SP_COLC, tl_launch_sp_col(0, c->blocksLA, c->smemSA, c->net, c->st, c->sc, c->tlA, s));
+    } else {
+        LAUNCH(c, s, CB_K_SP_ROWB, (k_sp_rowB_t<<<c->blocksTB, CB_THREADS, 0, s>>>(c->net, c->st, c->sc, c->tB)));
+        LAUNCH(c, s, CB_K_SP_COLC, (k_sp_colCA_t<<<c->blocksTA, CB_THREADS, 0, s>>>(c->net, c->st, c->sc, c->tA)));
+    }
     LAUNCH(c, s, CB_K_COUNTER, (k_advance<<<1, 32, 0, s>>>(c->st, c->sc, 1)));
     if (c->net.ball) LAUNCH(c, s, CB_K_BALL_X0, (k_ball_sp<<<c->net.S, CB_BALL_THREADS, 0, s>>>(c->net, c->st, 0)));
     if (c->opt.track_best)
@@ -1237,18 +1272,30 @@ static int sp_start(as_ctx* c) {
     LAUNCH(c, s, CB_K_SP_START, (k_sp_convert_elem<<<grid_for(NHS), CB_THREADS, 0, s>>>(c->net, c->st, c->sc,
                                                                                       (float)c->opt.sp_c_alpha,
                                                                                       (float)c->opt.sp_c_beta)));
-    LAUNCH(c, s, CB_K_SP_START, (k_sp_convert_P_t<<<c->blocksTA, CB_THREADS, 0, s>>>(c->net, c->st, c->sc, c->tA)));
+    if (c->sp_tiles) {
+        LAUNCH(c, s, CB_K_SP_START, (k_rowprep<<<grid_for(NHS), CB_THREADS, 0, s>>>(c->net, c->st, c->sc, 2)));
+        LAUNCH(c, s, CB_K_SP_START, tl_launch_sp_convert(c->blocksLA, c->smemLA, c->net, c->st, c->sc, c->tlA, s));
+    } else {
+        LAUNCH(c, s, CB_K_SP_START, (k_sp_convert_P_t<<<c->blocksTA, CB_THREADS, 0, s>>>(c->net, c->st, c->sc, c->tA)));
+    }
     LAUNCH(c, s, CB_K_SP_START, (k_sp_prep<<<grid_for(NHS), CB_THREADS, 0, s>>>(c->net, c->st)));
-    LAUNCH(c, s, CB_K_SP_START, (k_sp_colA_t<<<c->blocksTA, CB_THREADS, 0, s>>>(c->net, c->st, c->tA, 1)));
+    launch_sp_phaseA(c, s, CB_K_SP_START, true);
     if (c->net.ball) LAUNCH(c, s, CB_K_BALL_X0, (k_ball_sp<<<c->net.S, CB_BALL_THREADS, 0, s>>>(c->net, c->st, 1)));
     TRY(check_launch(c, "Saddle Point conversion"));
     for (int t = 0; t < c->opt.sp_init_steps; ++t) {
-        LAUNCH(c, s, CB_K_SPI_ROW, (k_spi_row_t<<<c->blocksTB, CB_THREADS, 0, s>>>(c->net, c->st, c->tB)));
-        LAUNCH(c, s, CB_K_SPI_COL, (k_spi_col_t<<<c->blocksTA, CB_THREADS, 0, s>>>(c->net, c->st, c->sc, c->tA)));
+        if (c->sp_tiles) {
+            LAUNCH(c, s, CB_K_SPI_ROW, tl_launch_spi_row(c->blocksLB, c->smemSB, c->net, c->st, c->tlB, s));
+            LAUNCH(c, s, CB_K_SPI_COL, tl_launch_sp_col(3, c->blocksLA, c->smemSA, c->net, c->st, c->sc, c->tlA, s));
+        } else {
+            LAUNCH(c, s, CB_K_SPI_ROW, (k_spi_row_t<<<c->blocksTB, CB_THREADS, 0, s>>>(c->net, c->st, c->tB)));
+            LAUNCH(c, s, CB_K_SPI_COL, (k_spi_col_t<<<c->blocksTA, CB_THREADS, 0, s>>>(c->net, c->st, c->sc, c->tA)));
+        }
         LAUNCH(c, s, CB_K_COUNTER, (k_advance<<<1, 32, 0, s>>>(c->st, c->sc, 2)));
         if (c->net.ball)
             LAUNCH(c, s, CB_K_BALL_X0, (k_ball_retract<<<c->net.S, CB_BALL_THREADS, 0, s>>>(c->net, c->st)));
     }
+    if (c->sp_tiles && c->opt.sp_init_steps > 0)   // alpha back into the output records
+        LAUNCH(c, s, CB_K_SP_START, (k_sp_prep<<<grid_for(NHS), CB_THREADS, 0, s>>>(c->net, c->st)));
     TRY(check_launch(c, "Saddle Point primal initialisation"));
     c->sp_started = true;
     c->sp_need_phaseA = true;
@@ -1262,7 +1309,7 @@ extern "C" int sp_step(as_ctx* c, int n_iters) {
     if (n_iters == 0) return AS_OK;
     if (c->sp_need_phaseA) {
         cudaStream_t s = c->stream;
-        LAUNCH(c, s, CB_K_SP_COLA, (k_sp_colA_t<<<c->blocksTA, CB_THREADS, 0, s>>>(c->net, c->st, c->tA, 0)));
+        launch_sp_phaseA(c, s, CB_K_SP_COLA, false);
         if (c->net.ball) LAUNCH(c, s, CB_K_BALL_X0, (k_ball_sp<<<c->net.S, CB_BALL_THREADS, 0, s>>>(c->net, c->st, 0)));
         TRY(check_launch(c, "Saddle Point phase A"));
         c->sp_need_phaseA = false;
@@ -1276,7 +1323,7 @@ extern "C" int as_bound(as_ctx* c, int precision, double* out, double* best) {
     const int S = c->net.S;
     cudaStream_t s = c->stream;
     if (c->sp_started) {
-        LAUNCH(c, s, CB_K_SP_COLA, (k_sp_colA_t<<<c->blocksTA, CB_THREADS, 0, s>>>(c->net, c->st, c->tA, 0)));
+        launch_sp_phaseA(c, s, CB_K_SP_COLA, false);
         if (c->net.ball) LAUNCH(c, s, CB_K_BALL_X0, (k_ball_sp<<<S, CB_BALL_THREADS, 0, s>>>(c->net, c->st, 0)));
     } else {
         // the BF16 form's iterates give a bound through float32 records (its lambda, kappa are float32)

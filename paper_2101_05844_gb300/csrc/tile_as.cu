@@ -312,6 +312,46 @@ __global__ void __launch_bounds__(CB_THREADS, 2) k_as_colA_tl(DNet net, DState s
     }
 }
 
+// Saddle Point's start (eq. 10): P_k = W^T beta_{k,1} + sum_b (W o I_b)^T beta_{k,b}, the col pass's masked
+// product over records that hold beta_1 in the place of -(alpha - beta_1) (k_rowprep).
+template <int NS>
+__device__ __forceinline__ void convert_tile(const DNet& net, const DState& st, const DLayer& L, const TlSegs& segs,
+                                             const TlSeg& g, const TlTile& t, int bo, char* smem) {
+    if (g.ch == 8) col_sums<NS, 8, ColOp<NS, 8>>(net, st, L, g, t, bo, smem);
+    else col_sums<NS, 4, ColOp<NS, 4>>(net, st, L, g, t, bo, smem);
+    const float* sums = reinterpret_cast<const float*>(smem);
+    if (g.ks > 1 && !tl_join<1>(segs, g, t, reinterpret_cast<float*>(smem))) return;
+    __syncthreads();
+    const int TC = tl_channels(g), row = tl_lanes(g) + 1;
+    for (int u = threadIdx.x; u < tl_units(g); u += CB_THREADS) {
+        int ch, lane, s, p;
+        tl_order(g, L.kind == 0, u, ch, lane);
+        if (!tl_unit(g, t, lane, net.S, s, p) || t.ct * TC + ch >= g.C) continue;
+        st.P[(size_t)s * net.NT + L.in_off + tl_col_neuron(L, g, t.ct * TC + ch, p)] = sums[ch * row + lane];
+    }
+}
+__global__ void __launch_bounds__(CB_THREADS, 2) k_sp_convert_tl(DNet net, DState st, DSched sc,
+                                                                 const __grid_constant__ TlSegs segs) {
+    extern __shared__ __align__(16) char tile_smem[];
+    const TlSeg& g = segs.s[tlseg_of(segs, blockIdx.x)];
+    if (!g.nch) return;   // the output layer's inputs carry no P
+    const DLayer& L = net.L[g.li];
+    const TlTile t = tl_tile(g);
+    const StepNow sp = cb_step(st);
+    const int bo = sp.nadd_before & 1;
+    switch (min(sp.nadd_before, sc.maxcut)) {
+        case 0: convert_tile<0>(net, st, L, segs, g, t, bo, tile_smem); break;
+        case 1: convert_tile<1>(net, st, L, segs, g, t, bo, tile_smem); break;
+        case 2: convert_tile<2>(net, st, L, segs, g, t, bo, tile_smem); break;
+        case 3: convert_tile<3>(net, st, L, segs, g, t, bo, tile_smem); break;
+        case 4: convert_tile<4>(net, st, L, segs, g, t, bo, tile_smem); break;
+        case 5: convert_tile<5>(net, st, L, segs, g, t, bo, tile_smem); break;
+        case 6: convert_tile<6>(net, st, L, segs, g, t, bo, tile_smem); break;
+        case 7: convert_tile<7>(net, st, L, segs, g, t, bo, tile_smem); break;
+        default: convert_tile<8>(net, st, L, segs, g, t, bo, tile_smem); break;
+    }
+}
+
 // ---------------------------------------------------------------- row pass
 // W x* and the masked products from the input records {x*, p bits | q bits << 8}: under a positive weight
 // a slot takes x* where its p bit is set, under a negative one where its q bit is. The records are
@@ -467,6 +507,7 @@ cudaError_t tl_as_prepare(int smem_col, int smem_row) {
     cudaError_t e = cudaFuncSetAttribute(k_as_colA_tl<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_col);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_as_colA_tl<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_col);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_sp_convert_tl, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_col);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_as_rowB_tl, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_row);
     return e;
 }
@@ -480,6 +521,11 @@ void tl_launch_colA(bool seq, int blocks, int smem, const DNet& net, const DStat
 void tl_launch_rowB(int blocks, int smem, const DNet& net, const DState& st, const DSched& sc, const TlSegs& t,
                     cudaStream_t s) {
     k_as_rowB_tl<<<blocks, CB_THREADS, smem, s>>>(net, st, sc, t);
+}
+
+void tl_launch_sp_convert(int blocks, int smem, const DNet& net, const DState& st, const DSched& sc, const TlSegs& t,
+                          cudaStream_t s) {
+    k_sp_convert_tl<<<blocks, CB_THREADS, smem, s>>>(net, st, sc, t);
 }
 
 }  // namespace cb
