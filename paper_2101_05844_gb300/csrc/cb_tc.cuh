@@ -28,6 +28,7 @@
 // after AS_ERR_TIMEOUT are void either way).
 #pragma once
 #include <cstdint>
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include "cb_common.cuh"
@@ -580,6 +581,150 @@ __global__ void __launch_bounds__(TC_THREADS) k_gemm_wgroup_bf16(GemmGroup gg, i
     const int M = group_rows(gg, g);
     if ((long long)blockIdx.x * (MT * TC_BM) >= M) return;
     win_tile<BN, MT>(gg.wa[g], gg.B[g], gg.ldb[g], gg.D[g], M, gg.N, gg.K[g], status, gg.stage_limit);
+}
+
+// Linear layers: both operands are dense K-major matrices (a row of A is a (slot, subproblem)), so the
+// tiles come by TMA in the 128-byte swizzled layout, through a ring of stages that one thread fills and one
+// thread empties with tcgen05.mma; the four warps meet for the epilogue. The gathered kernel above keeps one
+// K tile in flight and waits for each (81 us for 1536 x 1024 x 2048 at 32 columns a tile, of which the MMAs
+// take 4); it stays for the strided convolutions' row passes.
+struct TmaGemm {
+    float* D;                // [M][N] row-major
+    int M, N, K, rows_per_slot;
+    const int* ctr;
+    DSched sc;
+    int row_pass;
+    uint32_t stage_limit;
+};
+
+constexpr int TMA_STAGE_A = TC_BM * TC_BK * 2;
+template <int BN>
+__host__ __device__ constexpr int tma_stages() { return BN == 128 ? 6 : 4; }   // one CTA of 128 columns per SM, two narrower ones
+template <int BN>
+__host__ __device__ constexpr int tma_smem_bytes() { return tma_stages<BN>() * (TMA_STAGE_A + BN * TC_BK * 2) + 1024 + 256; }
+
+__device__ __forceinline__ void tma_load(uint32_t dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
+        "l"(map), "r"(x), "r"(y), "r"(smem_u32(bar))
+        : "memory");
+}
+__device__ __forceinline__ void mbar_expect(uint64_t* bar, uint32_t bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
+}
+// Descriptor of a K-major tile of 64 bf16 per row in the 128-byte swizzle: rows of 128 bytes, groups of
+// eight rows 1024 bytes apart; a K step of 16 starts 32 bytes further.
+__device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t addr) {
+    return static_cast<uint64_t>((addr >> 4) & 0x3FFFu) | (static_cast<uint64_t>(1u) << 16) |
+           (static_cast<uint64_t>(1024u >> 4) << 32) | (static_cast<uint64_t>(1u) << 46) | (static_cast<uint64_t>(2u) << 61);
+}
+
+template <int BN>
+__global__ void __launch_bounds__(TC_THREADS) k_gemm_tma_bf16(const __grid_constant__ CUtensorMap ma,
+                                                              const __grid_constant__ CUtensorMap mb, TmaGemm g,
+                                                              int* status) {
+    constexpr int ST = tma_stages<BN>(), STAGE = TMA_STAGE_A + BN * TC_BK * 2;
+    extern __shared__ uint8_t tma_raw[];
+    __shared__ uint64_t full[ST], empty[ST], done;
+    __shared__ uint32_t tslot;
+    __shared__ volatile int issued_s, consumed_s, stop_s;
+    // rows in use at the current iteration (as group_rows)
+    int M = g.M;
+    {
+        const int it = *g.ctr;
+        int ns = 0;
+        if (it >= g.sc.TM) {
+            const int t = it - g.sc.TM;
+            ns = cb_additions_before(t, g.sc);
+            if (g.row_pass && cb_slot_at(t, g.sc) >= 0) ++ns;
+            ns = min(ns, g.sc.maxcut);
+        }
+        M = (int)min((long long)M, (long long)(1 + ns) * g.rows_per_slot);
+    }
+    const int m0 = blockIdx.x * TC_BM, n0 = blockIdx.y * BN;
+    if (m0 >= M) return;   // the whole CTA, before any barrier
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const uint32_t base = (smem_u32(tma_raw) + 1023u) & ~1023u;
+    const int KT = (g.K + TC_BK - 1) / TC_BK;
+    if (warp == 0) tmem_alloc(&tslot, BN);
+    if (tid == 0) {
+        for (int s = 0; s < ST; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 1);
+        }
+        mbar_init(&done, 1);
+        issued_s = consumed_s = stop_s = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = tslot;
+    if (tid == 0) {   // fills the stages
+        int kt = 0;
+        for (; kt < KT; ++kt) {
+            const int s = kt % ST;
+            if (kt >= ST && !mbar_wait(&empty[s], ((kt / ST) - 1) & 1u, g.stage_limit)) break;
+            if (stop_s) break;
+            const uint32_t a = base + s * STAGE;
+            mbar_expect(&full[s], STAGE);
+            tma_load(a, &ma, kt * TC_BK, m0, &full[s]);
+#pragma unroll
+            for (int q = 0; q < BN / 32; ++q)
+                tma_load(a + TMA_STAGE_A + q * 32 * TC_BK * 2, &mb, kt * TC_BK, n0 + q * 32, &full[s]);
+        }
+        issued_s = kt;
+    } else if (tid == 32) {   // empties them
+        constexpr uint32_t idesc = idesc_bf16(TC_BM, BN);
+        int kt = 0;
+        for (; kt < KT; ++kt) {
+            const int s = kt % ST;
+            if (!mbar_wait(&full[s], (kt / ST) & 1u, g.stage_limit)) {
+                stop_s = 1;
+                break;
+            }
+            tc_fence_after();
+            const uint32_t a = base + s * STAGE, b = a + TMA_STAGE_A;
+#pragma unroll
+            for (int kk = 0; kk < TC_BK / 16; ++kk)
+                mma_bf16(tmem, smem_desc_sw128(a + kk * 32), smem_desc_sw128(b + kk * 32), idesc, (kt > 0 || kk > 0) ? 1u : 0u);
+            mma_commit(&empty[s]);
+        }
+        mma_commit(&done);
+        consumed_s = kt;
+    }
+    __syncthreads();
+    // a wait that ran out leaves loads in flight: they land before the CTA goes
+    bool f_ok = true;
+    if (tid == 0)
+        for (int kt = consumed_s; kt < issued_s; ++kt) f_ok = mbar_wait(&full[kt % ST], (kt / ST) & 1u) && f_ok;
+    f_ok = mbar_wait(&done, 0u) && f_ok;
+    const bool drained = __syncthreads_and(f_ok);
+    const bool ok = drained && consumed_s == KT;
+    if (!ok && tid == 0 && status) atomicExch(status, TC_ERR_TIMEOUT);
+    tc_fence_after();
+    if (ok) {
+        const int row = m0 + warp * 32 + lane;
+#pragma unroll 1
+        for (int c0 = 0; c0 < BN; c0 += 16) {
+            float v[16];
+            tmem_ld16(tmem + (static_cast<uint32_t>(warp * 32) << 16) + c0, v);
+            if (row >= M || n0 + c0 >= g.N) continue;
+            float* dr = g.D + (size_t)row * g.N + n0 + c0;
+            if (n0 + c0 + 16 <= g.N && (g.N & 3) == 0) {
+#pragma unroll
+                for (int j = 0; j < 16; j += 4)
+                    *reinterpret_cast<float4*>(dr + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+            } else {
+#pragma unroll
+                for (int j = 0; j < 16; ++j)
+                    if (n0 + c0 + j < g.N) dr[j] = v[j];
+            }
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 0 && drained) tmem_free(tmem, BN);
 }
 
 }  // namespace tc

@@ -71,6 +71,8 @@ struct as_ctx {
         tc::GemmGroup g;
         int ng, maxM, bn;
         int win = 0, mt = 1, smem = 0;   // window operands (k_gemm_wgroup_bf16): row blocks per CTA, bytes
+        int tma = 0;                     // dense operands by TMA (k_gemm_tma_bf16): linear layers
+        CUtensorMap ma, mb;
     };
     std::vector<TcGemm> tc_row, tc_col;           // per hidden-output layer
     std::vector<TcGemm> tc_row_alt, tc_col_alt;   // gathered-operand plans beside window ones (autotune)

@@ -132,3 +132,29 @@ def test_tiles_agree_with_lane_teams(name, S, nslots, add, ball):
             bad = off > RTOL * (np.abs(b) + np.abs(b).max() + 1e-6)
             # a choice (eq. 12) within rounding of a tie may fall the other way
             assert bad.mean() < 2e-3, (name, steps, w, bad.mean(), off.max())
+
+
+@pytest.mark.parametrize("widths,S,nslots", [((100, 75, 33, 7), 129, 3), ((300, 130, 257, 4), 300, 0), ((520, 40, 64, 3), 41, 5)])
+def test_bf16_linear_products_do_not_depend_on_their_tiles(widths, S, nslots):
+    """The BF16 form's dense products (TMA, 128, 64 or 32 columns a tile): rows, columns and K that fill no
+    tile. The K order of the sums is the tiles' same, so a batch (wide tiles) and each of its subproblems
+    alone (narrow ones) agree bit for bit; against the oracle, test_gpu_bf16.py checks small ones."""
+    net = synth.make_net(synth._mlp(list(widths)), 7)
+    c, lo, hi = synth.make_boxes(widths[0], S, 0.05, 8)
+    C = synth.properties_runner_up(synth.forward(net, c))
+    cap = max(1, nslots)
+    kw = dict(bigm_iters=10, as_iters=1000, omega=0, vars_per_add=cap, max_cuts=cap, graph_chunk=0, precision=16)
+    big = binding.Context(net, lo, hi, C, options=binding.default_options(**kw))
+    d = _draw(big, np.random.default_rng(9), S, nslots, 110 if nslots else 3, cap)
+    outs = [binding.ST_ALPHA, binding.ST_BETA0, binding.ST_BETA1, binding.ST_SLOT_BETA]
+    for w, v in d.items():
+        big.set_state(w, v)
+    big.as_step(2)
+    for s in (0, S // 2, S - 1):
+        one = binding.Context(net, lo[s:s + 1], hi[s:s + 1], C[s:s + 1], options=binding.default_options(**kw))
+        for w, v in d.items():
+            one.set_state(w, v if w == binding.ST_ITER else np.take(v, [s], _axis(w)))
+        one.as_step(2)
+        for w in outs:
+            a = np.take(big.get_state(w).reshape(d[w].shape), [s], _axis(w))
+            np.testing.assert_array_equal(a.ravel(), one.get_state(w))
