@@ -290,7 +290,7 @@ __device__ __forceinline__ int tl_col_neuron(const DLayer& L, const TlSeg& g, in
 }
 
 // Launches (tile_as.cu). tl_weights fills a segment's weights from its layer's; tl_as_prepare allows
-// the passes their shared memory; the col pass takes the bound's evaluation (seq) in the lane teams' order.
+// the passes their shared memory; seq: the col pass's sums in the lane teams' order.
 void tl_weights(const DLayer& L, bool col, const TlSeg& g, float* w, float2* wpm, cudaStream_t s);
 cudaError_t tl_as_prepare(int smem_col, int smem_row);
 void tl_launch_colA(bool seq, int blocks, int smem, const DNet& net, const DState& st, const DSched& sc, const TlSegs& t,

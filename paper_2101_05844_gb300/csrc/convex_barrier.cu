@@ -1158,12 +1158,12 @@ extern "C" void as_destroy(as_ctx* c) {
 }
 
 // ------------------------------------------------------------------------------- iterations
-// The float32 col pass: the tiled layers, then the lane teams' share. Mode 1 (the bound's evaluation
-// at the current duals) takes the sums in the lane teams' order.
-static void launch_colA(as_ctx* c, cudaStream_t s, int mode) {
+// The float32 col pass: the tiled layers, then the lane teams' share; seq: the tiles' sums in the lane
+// teams' order.
+static void launch_colA(as_ctx* c, cudaStream_t s, int mode, bool seq) {
     if (c->blocksLA)
         LAUNCH(c, s, CB_K_AS_COLA,
-               tl_launch_colA(mode == 1, c->blocksLA, c->smemLA, c->net, c->st, c->sc, c->tlA, mode, s));
+               tl_launch_colA(seq, c->blocksLA, c->smemLA, c->net, c->st, c->sc, c->tlA, mode, s));
     if (c->blocksTAr)
         LAUNCH(c, s, CB_K_AS_COLA,
                (k_as_colA_t<false><<<c->blocksTAr, CB_THREADS, 0, s>>>(c->net, c->st, c->sc, c->tAr, mode)));
@@ -1172,14 +1172,15 @@ static void launch_colA(as_ctx* c, cudaStream_t s, int mode) {
 static int launch_as_iter(as_ctx* c, cudaStream_t s) {
     // the per-neuron bound terms are only summed when the best bound is tracked
     const int mode = c->opt.track_best ? 0 : 2;
-    launch_colA(c, s, mode);
+    launch_colA(c, s, mode, false);
     if (c->net.ball) LAUNCH(c, s, CB_K_BALL_X0, (k_ball_x0<<<c->net.S, CB_BALL_THREADS, 0, s>>>(c->net, c->st)));
     if (c->opt.track_best)
         LAUNCH(c, s, CB_K_REDUCE, (k_reduce<<<c->net.S, CB_THREADS, 0, s>>>(c->net, c->st, 64, nullptr, 1)));
     if (c->blocksLB)
         LAUNCH(c, s, CB_K_AS_ROWB, tl_launch_rowB(c->blocksLB, c->smemLB, c->net, c->st, c->sc, c->tlB, s));
     if (c->blocksTBr)
-        LAUNCH(c, s, CB_K_AS_ROWB, (k_as_rowB_t<false><<<c->blocksTBr, CB_THREADS, 0, s>>>(c->net, c->st, c->sc, c->tBr)));
+        LAUNCH(c, s, CB_K_AS_ROWB,
+               (k_as_rowB_t<false><<<c->blocksTBr, CB_THREADS, 0, s>>>(c->net, c->st, c->sc, c->tBr)));
     LAUNCH(c, s, CB_K_COUNTER, (k_advance<<<1, 32, 0, s>>>(c->st, c->sc, 0)));
     return check_launch(c, "Active Set iteration");
 }
@@ -1330,7 +1331,7 @@ extern "C" int as_bound(as_ctx* c, int precision, double* out, double* best) {
     } else {
         // the BF16 form's iterates give a bound through float32 records (its lambda, kappa are float32)
         if (c->opt.precision == 16) TRY(float_records(c));
-        launch_colA(c, s, 1);
+        launch_colA(c, s, 1, false);
         if (c->net.ball) LAUNCH(c, s, CB_K_BALL_X0, (k_ball_x0<<<S, CB_BALL_THREADS, 0, s>>>(c->net, c->st)));
     }
     double* dout = c->bound_out;

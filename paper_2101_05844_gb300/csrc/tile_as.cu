@@ -153,8 +153,9 @@ struct ColOp : ColRecords<NS> {
 
 // The same sums in the order of a lane per unit (cb_team.cuh): the positive taps of a channel, then its
 // negative ones, into one accumulator of the unmasked product. Two sweeps over the taps for every four
-// channels, for the evaluations whose x* must not depend on which walk found it (the bound and its
-// gradient).
+// channels, for the gradient, whose x* must not depend on which walk found it (an input at a tie of f moves
+// it; the bound is continuous there and takes the packed sums: 16.2 against 8.9 ms at 1024 conv4 boxes and
+// five slots).
 template <int NS, int CH>
 struct ColSeqOp : ColRecords<NS> {
     static constexpr int WB = 4, CW = 4, SWEEPS = 2 * CH / CW;
