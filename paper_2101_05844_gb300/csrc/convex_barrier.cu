@@ -15,6 +15,7 @@
 #include "cb_backward.cuh"
 #include "cb_team.cuh"
 #include "cb_tile.cuh"
+#include "cb_vec.cuh"
 #include "cb_tc.cuh"
 
 using namespace cb;
@@ -80,6 +81,8 @@ struct as_ctx {
     int* tc_status = nullptr;                     // set by a tensor-core kernel whose wait ran out
     TSegs tA1{}, tB1{};                           // one lane per unit
     int blocksTA1 = 0, blocksTB1 = 0;
+    VSegs vA{}, vB{};                             // layers with four neurons per thread
+    int blocksVA = 0, blocksVB = 0;
     long long team_row = 40000, team_col = 40000; // team-size targets of the float32 passes
     uint32_t tc_stage_limit = tc::TC_WAIT_LIMIT;  // try_wait rounds of the GEMMs' stage waits
     // conv products of the BF16 form by window operands where their taps are shifts of one grid

@@ -158,3 +158,37 @@ def test_bf16_linear_products_do_not_depend_on_their_tiles(widths, S, nslots):
         for w in outs:
             a = np.take(big.get_state(w).reshape(d[w].shape), [s], _axis(w))
             np.testing.assert_array_equal(a.ravel(), one.get_state(w))
+
+
+@pytest.mark.parametrize("nslots,add,ball", [(0, False, 0), (3, True, 0), (5, False, 1), (8, False, 0)])
+def test_bf16_passes_by_fours_equal_one_neuron_per_thread(nslots, add, ball):
+    """The BF16 form's passes with four neurons per thread (aligned offsets) against one per thread: the same
+    net with one more hidden neuron, of zero weights, has no aligned offsets; everything else is the same sums in
+    the same order, which the compiler may contract into fused multiply-adds differently: a few units in the
+    last place. Stride 1 and 2, channels that are no multiple of eight, several blocks of positions."""
+    layers = synth._convnet((3, 12, 20), [(9, 3, 1, 1), (8, 4, 2, 1)], [24, 3])
+    net = synth.make_net(layers, 11)
+    S, last = 5, net[-2]["n_out"]
+    wide = [dict(L) for L in net]
+    wide[-2] = dict(net[-2], n_out=last + 1, W=np.vstack([net[-2]["W"], np.zeros((1, net[-2]["n_in"]), np.float32)]),
+                    b=np.append(net[-2]["b"], np.float32(0)))
+    wide[-1] = dict(net[-1], n_in=last + 1, W=np.hstack([net[-1]["W"], np.zeros((net[-1]["n_out"], 1), np.float32)]))
+    c, lo, hi = synth.make_boxes(net[0]["n_in"], S, 0.05, 12)
+    C = synth.properties_runner_up(synth.forward(net, c))
+    cap = nslots + (1 if add else 0) or 1
+    caps = np.array([cap, max(1, cap - 1), cap, 1, cap], np.int32)
+    kw = dict(bigm_iters=10, as_iters=1000, omega=0, vars_per_add=cap, max_cuts=cap, graph_chunk=0, precision=16, input_l2=ball)
+    a = binding.Context(net, lo, hi, C, caps=caps, options=binding.default_options(**kw))
+    b = binding.Context(wide, lo, hi, C, caps=caps, options=binding.default_options(**kw))
+    d = _draw(a, np.random.default_rng(13), S, nslots, 10 + nslots if add else 10 + 100 if nslots else 3, cap)
+    for w, v in d.items():
+        a.set_state(w, v)
+        b.set_state(w, v if w == binding.ST_ITER else np.concatenate([v, np.zeros_like(v[..., :1])], -1))
+    a.as_step(2)
+    b.as_step(2)
+    for w in (binding.ST_ALPHA, binding.ST_BETA0, binding.ST_BETA1, binding.ST_SLOT_BETA, binding.ST_ADAM):
+        x = b.get_state(w).reshape(*d[w].shape[:-1], -1)[..., :-1]
+        y = a.get_state(w).reshape(d[w].shape)
+        bad = np.abs(x - y) > 2.0 ** -20 * (np.abs(x) + np.abs(x).max())
+        assert bad.mean() < 1e-3, (w, bad.mean())   # an input within rounding of a tie may move its rows
+    np.testing.assert_allclose(a.bound(64), b.bound(64), rtol=1e-6)
