@@ -192,14 +192,34 @@ __device__ inline void cb_set_step(int it, const DSched& d, const DState& st, in
     s->ib = make_float2(inv_bias_corr(st.bc1_tab, d.ntab, it + 1, d.b1), inv_bias_corr(st.bc2_tab, d.ntab, it + 1, d.b2));
 }
 
-// The schedule's scalars (no pass writes them) and a slot's bias corrections.
+// Small batches launch their passes so that a pass is resident before the one before it has ended
+// (launch_after on the host): it may start once every block of that one has, and waits here for all of its
+// memory. First statement of such a kernel.
+__device__ __forceinline__ void cb_after_previous() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// The schedule's scalars and a slot's bias corrections. Volatile loads: the launch before may write them,
+// and an invariant load (__ldg) could move above the wait for it.
 struct StepNow {
     int it, as_phase, t, b_new, nadd_before;
     float lr;
 };
+__device__ __forceinline__ int cb_load(const int* p) {
+    int v;
+    asm volatile("ld.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ float2 cb_load(const float2* p) {
+    float2 v;
+    asm volatile("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p) : "memory");
+    return v;
+}
 __device__ __forceinline__ StepNow cb_step(const DState& st) {
     const Step* s = st.step;
-    return {__ldg(&s->it), __ldg(&s->as_phase), __ldg(&s->t), __ldg(&s->b_new), __ldg(&s->nadd_before), __ldg(&s->lr)};
+    return {cb_load(&s->it), cb_load(&s->as_phase), cb_load(&s->t), cb_load(&s->b_new), cb_load(&s->nadd_before),
+            __int_as_float(cb_load(reinterpret_cast<const int*>(&s->lr)))};
 }
-__device__ __forceinline__ float2 cb_bias(const DState& st) { return __ldg(&st.step->ib); }
-__device__ __forceinline__ float2 cb_slot_bias(const DState& st, int b) { return __ldg(&st.step->sib[b]); }
+__device__ __forceinline__ float2 cb_bias(const DState& st) { return cb_load(&st.step->ib); }
+__device__ __forceinline__ float2 cb_slot_bias(const DState& st, int b) { return cb_load(&st.step->sib[b]); }

@@ -18,6 +18,7 @@ namespace cb {
 // after the launch that completes an iteration, and with the Active Set's the schedule: stream order
 // has every block of that launch done before it, and the next launches read the new values. One warp.
 __global__ void k_advance(DState st, DSched sc, int i) {
+    cb_after_previous();
     const int v = st.ctr[i] + 1;
     __syncwarp();
     if (threadIdx.x == 0) st.ctr[i] = v;
@@ -178,6 +179,7 @@ __global__ void k_fold(DNet net, const float* Wlast, const float* blast, const f
 // d[s] = bout[s] + sum of the per-neuron terms (eq. 6), in a fixed order (deterministic).
 // precision 64: FP64 sum; 32: float32 sum. keep_best: best[s] = max(best[s], d[s]).
 __global__ void k_reduce(DNet net, DState st, int precision, double* out, int keep_best) {
+    cb_after_previous();
     const int s = blockIdx.x;
     const double* t = st.terms + (size_t)s * net.NT;
     __shared__ double sd[CB_THREADS];

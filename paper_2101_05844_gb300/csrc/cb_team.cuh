@@ -476,6 +476,7 @@ __device__ __forceinline__ int tseg_of(const TSegs& sg, int blk) {
 template <bool TC>
 __global__ void __launch_bounds__(CB_THREADS, 4) k_as_colA_t(DNet net, DState st, DSched sc, TSegs sg,
                                                                        int mode) {
+    cb_after_previous();
     const int q = tseg_of(sg, blockIdx.x);
     const int li = sg.layer[q];
     const DLayer& L = net.L[li];
@@ -803,6 +804,7 @@ __device__ __forceinline__ void as_rowB_tc(const DNet& net, const DState& st, co
 
 template <bool TC>
 __global__ void __launch_bounds__(CB_THREADS, 4) k_as_rowB_t(DNet net, DState st, DSched sc, TSegs sg) {
+    cb_after_previous();
     const int q = tseg_of(sg, blockIdx.x);
     const DLayer& L = net.L[sg.layer[q]];
     const int T = sg.T[q];
@@ -1160,6 +1162,7 @@ __global__ void __launch_bounds__(CB_THREADS) k_sp_colA_t(DNet net, DState st, T
 // gradients alpha_bar (eq. 11) and beta_bar (eq. 12), the convex combination of alpha, Sb, G, C
 // (Alg. 2), and the output record for phase C and the next phase A.
 __global__ void __launch_bounds__(CB_THREADS) k_sp_rowB_t(DNet net, DState st, DSched sc, TSegs sg) {
+    cb_after_previous();
     const int q = tseg_of(sg, blockIdx.x);
     const DLayer& L = net.L[sg.layer[q]];
     const Unit u = team_unit(sg, q, L.n_out, net.S);
@@ -1222,6 +1225,7 @@ __global__ void __launch_bounds__(CB_THREADS) k_sp_rowB_t(DNet net, DState st, D
 // P_k and of the primal iterate (x_m, z_m) into the other buffer (Alg. 2), then runs phase A at
 // the new iterate. The launch after it (k_advance) advances the iteration counter.
 __global__ void __launch_bounds__(CB_THREADS) k_sp_colCA_t(DNet net, DState st, DSched sc, TSegs sg) {
+    cb_after_previous();
     const int q = tseg_of(sg, blockIdx.x);
     const int li = sg.layer[q];
     const DLayer& L = net.L[li];
