@@ -427,12 +427,13 @@ __device__ __forceinline__ void sp_phaseA_epilogue(const DNet& net, const DState
 
 // Phase B of one row after its sums (a0 = W x, A = (W o I*) x, Lam, Mu the row sums of the oracle mask,
 // nout its unselected free inputs): conditional gradients alpha_bar (eq. 11) and beta_bar (eq. 12), the
-// convex combination of alpha, Sb, G, C at iteration t, and the output record.
+// convex combination of alpha, Sb, G, C at iteration t, and the output record. h: the row's index in a hidden
+// vector, z its primal value (worked out again here, the lane teams' kernel took 64 registers instead of 48: 25
+// iterations on the Wide conv net's nine properties 1500 us instead of 1473).
 __device__ __forceinline__ void sp_rowB_unit(const DNet& net, const DState& st, const DSched& sc, const DLayer& L, int s,
-                                             int i, int t, float a0, float A, float Lam, float Mu, int nout) {
+                                             int i, size_t h, int t, float z, float a0, float A, float Lam, float Mu, int nout) {
     const int cur = t & 1;
-    const size_t NT = net.NT, h = (size_t)s * net.NH + L.h_out + i;
-    const float z = st.spz[cur][h];
+    const size_t NT = net.NT;
     // a row selecting none or all of its free inputs is the all-zero / all-ones constraint, a
     // looser copy of beta_0 / beta_1: it does not compete in the choice of eq. (12)
     const bool degenerate = nout == 0 || nout == st.nfree[h];

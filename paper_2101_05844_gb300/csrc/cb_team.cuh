@@ -1215,7 +1215,7 @@ __global__ void __launch_bounds__(CB_THREADS) k_sp_rowB_t(DNet net, DState st, D
         for (int o = u.T >> 1; o > 0; o >>= 1) nout += __shfl_xor_sync(0xffffffffu, nout, o);
     }
     if (!u.valid || u.lane != 0) return;
-    sp_rowB_unit(net, st, sc, L, s, i, t, a0, A, Lam, Mu, nout);
+    sp_rowB_unit(net, st, sc, L, s, i, h, t, z, a0, A, Lam, Mu, nout);
 }
 
 // Phase C of iteration t fused with phase A of iteration t + 1 (col pass over k = 1..n): one walk

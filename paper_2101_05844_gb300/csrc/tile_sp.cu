@@ -212,7 +212,9 @@ __device__ __forceinline__ void sp_row_tile(const DNet& net, const DState& st, c
         if (!tl_unit(g, t, lane, net.S, s, p) || t.ct * TC + ch >= g.C) continue;
         const float* v = sums + ch * row + lane;
         const int n = TC * row;
-        sp_rowB_unit(net, st, sc, L, s, (t.ct * TC + ch) * g.P + p, it, v[0], v[n], v[2 * n], v[3 * n], (int)v[4 * n]);
+        const int i = (t.ct * TC + ch) * g.P + p;
+        const size_t h = (size_t)s * net.NH + L.h_out + i;
+        sp_rowB_unit(net, st, sc, L, s, i, h, it, st.spz[it & 1][h], v[0], v[n], v[2 * n], v[3 * n], (int)v[4 * n]);
     }
 }
 __global__ void __launch_bounds__(CB_THREADS, 2) k_sp_rowB_tl(DNet net, DState st, DSched sc,
