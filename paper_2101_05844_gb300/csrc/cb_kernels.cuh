@@ -98,13 +98,14 @@ __global__ void k_ibp(DNet net, DState st, int li, const signed char* splits) {
     }
 }
 
-// A batch's start: no best bound yet, the schedule of iteration 0 (the counters have been cleared).
-__global__ void k_start(DState st, DSched sc, int S) {
+// A batch's start: no best bound yet, the schedule of iteration 0 (the counters have been cleared), and with
+// `caps` every subproblem's cap.
+__global__ void k_start(DState st, DSched sc, int S, int* caps, int cap) {
     if (blockIdx.x == 0 && threadIdx.x < 32) cb_set_step(0, sc, st, threadIdx.x);
-    for (int u = blockIdx.x * blockDim.x + threadIdx.x; u < S; u += gridDim.x * blockDim.x) st.best[u] = -INFINITY;
-}
-__global__ void k_fill_int(int* p, size_t n, int v) {
-    for (size_t u = blockIdx.x * (size_t)blockDim.x + threadIdx.x; u < n; u += (size_t)gridDim.x * blockDim.x) p[u] = v;
+    for (int u = blockIdx.x * blockDim.x + threadIdx.x; u < S; u += gridDim.x * blockDim.x) {
+        st.best[u] = -INFINITY;
+        if (caps) caps[u] = cap;
+    }
 }
 
 // Device-side check of a box given on the device: sets the status word if lo > hi or non-finite.

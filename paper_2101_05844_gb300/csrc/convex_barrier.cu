@@ -855,7 +855,7 @@ static int load_batch(as_ctx* c, const float* x_lo, const float* x_hi, const flo
     TRY(clear_planes(c));
     c->bounds_ibp = lhat == nullptr;
     c->have_splits = splits != nullptr && lhat == nullptr;
-    LAUNCH(c, s, CB_K_BATCH, (k_start<<<grid_for(S), CB_THREADS, 0, s>>>(st, c->sc, S)));
+    LAUNCH(c, s, CB_K_BATCH, (k_start<<<grid_for(S), CB_THREADS, 0, s>>>(st, c->sc, S, caps ? nullptr : c->caps_dev, c->opt.max_cuts)));
     c->sp_started = false;
     if (host_checks) {
         std::vector<float> hl((size_t)S * n0), hh((size_t)S * n0);
@@ -883,9 +883,6 @@ static int load_batch(as_ctx* c, const float* x_lo, const float* x_hi, const flo
         LAUNCH(c, s, CB_K_BATCH, (k_check_box<<<grid_for((size_t)S * n0), CB_THREADS, 0, s>>>(D, st)));
     }
     if (caps) CUDA_TRY(c, cudaMemcpyAsync(c->caps_dev, caps, S * sizeof(int), cudaMemcpyDefault, s));
-    else {
-        LAUNCH(c, s, CB_K_BATCH, (k_fill_int<<<grid_for(S), CB_THREADS, 0, s>>>(c->caps_dev, (size_t)S, c->opt.max_cuts)));
-    }
     if (C) CUDA_TRY(c, cudaMemcpyAsync(c->C, C, (size_t)S * c->n_out * sizeof(float), cudaMemcpyDefault, s));
     LAUNCH(c, s, CB_K_BATCH, (k_fold<<<S, CB_THREADS, 0, s>>>(D, c->Wlast, c->blast, C ? c->C : nullptr, c->n_out,
                                                              (float*)D.Wout, (float*)D.bout)));
