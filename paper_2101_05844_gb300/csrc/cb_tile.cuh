@@ -232,16 +232,23 @@ __device__ __forceinline__ void tl_put(const TlSeg& g, const TlTile& t, float* s
         for (int e = 0; e < NV; ++e) sums[(e * TC + t.c0 + c) * row + t.lane] = v[c][e];
 }
 
-// A split tile: this block's sums into the scratch; true in the block that arrives last, which then
-// holds the tile's sums (added in split order). Every thread takes part.
+// A split tile's partial sums in the scratch.
 template <int NV>
-__device__ __forceinline__ bool tl_join(const TlSegs& segs, const TlSeg& g, const TlTile& t, float* sums) {
+__device__ __forceinline__ float4* tl_partials(const TlSegs& segs, const TlSeg& g, const TlTile& t) {
+    return reinterpret_cast<float4*>(segs.part + g.part) + (size_t)t.tile * g.ks * (tl_split(g, NV) / 4);
+}
+
+// This block's sums into the scratch; true in the block that arrives last, which then sees every split's.
+// Every thread takes part.
+template <int NV>
+__device__ __forceinline__ bool tl_arrive(const TlSegs& segs, const TlSeg& g, const TlTile& t, const float* sums) {
     const int n4 = (NV * tl_channels(g) * (tl_lanes(g) + 1) + 3) / 4;
     const size_t stride = tl_split(g, NV) / 4;
-    float4* part = reinterpret_cast<float4*>(segs.part + g.part) + (size_t)t.tile * g.ks * stride;
+    float4* part = tl_partials<NV>(segs, g, t);
     __shared__ int last;
     __syncthreads();
-    for (int i = threadIdx.x; i < n4; i += CB_THREADS) __stcg(part + t.ks * stride + i, reinterpret_cast<float4*>(sums)[i]);
+    for (int i = threadIdx.x; i < n4; i += CB_THREADS)
+        __stcg(part + t.ks * stride + i, reinterpret_cast<const float4*>(sums)[i]);
     __threadfence();
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -252,6 +259,16 @@ __device__ __forceinline__ bool tl_join(const TlSegs& segs, const TlSeg& g, cons
     __syncthreads();
     if (!last) return false;
     __threadfence();
+    return true;
+}
+
+// A split tile: true in the block that arrives last, which then holds the tile's sums (added in split order).
+template <int NV>
+__device__ __forceinline__ bool tl_join(const TlSegs& segs, const TlSeg& g, const TlTile& t, float* sums) {
+    if (!tl_arrive<NV>(segs, g, t, sums)) return false;
+    const int n4 = (NV * tl_channels(g) * (tl_lanes(g) + 1) + 3) / 4;
+    const size_t stride = tl_split(g, NV) / 4;
+    const float4* part = tl_partials<NV>(segs, g, t);
     for (int i = threadIdx.x; i < n4; i += CB_THREADS) {
         float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
         for (int q = 0; q < g.ks; q += 8) {   // eight splits in flight
@@ -299,9 +316,10 @@ void tl_launch_rowB(int blocks, int smem, const DNet& net, const DState& st, con
                     cudaStream_t s);
 // Interval propagation (tile_sp.cu): the input box's records, then a row segment per hidden layer.
 int tl_ibp_smem(const TlSeg& g);
+int tl_ibp_splits(const TlSeg& g, int S);
 cudaError_t tl_sp_prepare(int smem_ibp, int smem_row, int smem_col);
 void tl_launch_ibp_box(int grid, const DNet& net, const DState& st, cudaStream_t s);
-void tl_launch_ibp(const DNet& net, const DState& st, const TlSeg& seg, const signed char* splits, cudaStream_t s);
+void tl_launch_ibp(const DNet& net, const DState& st, const TlSegs& segs, int q, const signed char* splits, cudaStream_t s);
 // Saddle Point (tile_sp.cu): its passes, the col pass's work by `what` (0: phase C and the next phase A, 1:
 // phase A, 2: phase A starting the primal iterate, 3: a step of the primal initialisation).
 int tl_sp_row_smem(const TlSeg& g);

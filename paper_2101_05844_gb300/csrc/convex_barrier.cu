@@ -546,6 +546,14 @@ static int build_tiles(as_ctx* c, const std::vector<std::vector<float>>& Wh) {
     // (scratch and shared memory also serve Saddle Point's passes on the same tiles: 2 and 5 values per unit)
     TRY(finish(pa, c->tlA, c->blocksLA, c->smemLA, true));
     TRY(finish(pb, c->tlB, c->blocksLB, c->smemLB, false));
+    // interval propagation splits its layers by a rule of its own
+    for (int q = 0; q < c->tlB.n && c->tlB.n == n - 1 && !D.ball; ++q) {
+        const TlSeg& g = c->tlB.s[q];
+        const int ks = tl_ibp_splits(g, S);
+        if (ks == 1) continue;
+        part = std::max(part, (size_t)tl_tiles(g, S) * ks * tl_split(g, 5));
+        ctrs = std::max(ctrs, tl_tiles(g, S));
+    }
     if (ctrs) {
         TRY(dalloc(c, &c->tlA.part, part));
         TRY(dalloc(c, &c->tlA.ctr, (size_t)ctrs));
@@ -914,7 +922,7 @@ static int load_batch(as_ctx* c, const float* x_lo, const float* x_hi, const flo
             const long long warps = (long long)S * D.L[k].n_out;
             if (tiled && !D.ball) {
                 for (int q = 0; q < c->tlB.n; ++q)
-                    if (c->tlB.s[q].li == k) LAUNCH(c, s, CB_K_BATCH, tl_launch_ibp(D, st, c->tlB.s[q], dsp, s));
+                    if (c->tlB.s[q].li == k) LAUNCH(c, s, CB_K_BATCH, tl_launch_ibp(D, st, c->tlB, q, dsp, s));
                 TRY(check_launch(c, "k_ibp_tl"));
                 continue;
             }

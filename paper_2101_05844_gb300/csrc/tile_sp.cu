@@ -10,7 +10,8 @@ namespace cb {
 // by compensated float32 sums (CompSum: float64 accuracy), from records {l, u} of the layer's inputs
 // kept in the first Saddle Point input plane. A warp per row (k_ibp) reads every weight and bound of a
 // row from L1 for that row alone: 26.6 ms for 256 conv4 boxes, where the sums' 20 operations per tap take
-// about 1.6 ms at the float32 rate.
+// about 1.6 ms at the float32 rate. On tiles 4.5 ms, and 4.0 with the layers of few tiles split over their
+// sources (tl_ibp_splits).
 template <int CH>
 struct IbpOp {
     static constexpr int RB = 8, EB = 0, WB = 4, SWEEPS = 1;
@@ -81,19 +82,37 @@ __device__ __forceinline__ void ibp_tile(const DNet& net, const DState& st, cons
         }
         tl_put<5, CH>(g, t, sums, v);
     }
+    // the splits' pairs of a row are added in float64 by the block that arrives last
+    if (g.ks > 1 && !tl_arrive<5>(segs, g, t, sums)) return;
     __syncthreads();
     const int TC = tl_channels(g), row = tl_lanes(g) + 1;
+    const float* part = reinterpret_cast<const float*>(tl_partials<5>(segs, g, t));
     for (int u = threadIdx.x; u < tl_units(g); u += CB_THREADS) {
         int ch, lane, s, p;
         tl_order(g, L.kind == 0, u, ch, lane);
         if (!tl_unit(g, t, lane, net.S, s, p) || t.ct * TC + ch >= g.C) continue;
         const int i = (t.ct * TC + ch) * g.P + p, at = ch * row + lane;
-        auto val = [&](int e) { return sums[e * TC * row + at]; };
-        double a = (double)val(0) + (double)val(1), c = (double)val(2) + (double)val(3);
+        double a = 0.0, c = 0.0;
+        int nf = 0;
+        if (g.ks == 1) {
+            auto val = [&](int e) { return sums[e * TC * row + at]; };
+            a = (double)val(0) + (double)val(1);
+            c = (double)val(2) + (double)val(3);
+            nf = __float_as_int(val(4));
+        } else {
+#pragma unroll 4
+            for (int q = 0; q < g.ks; ++q) {
+                const float* v = part + q * tl_split(g, 5) + at;
+                auto val = [&](int e) { return __ldcg(v + e * TC * row); };
+                a += (double)val(0) + (double)val(1);
+                c += (double)val(2) + (double)val(3);
+                nf += __float_as_int(val(4));
+            }
+        }
         const size_t h = (size_t)s * net.NH + L.h_out + i;
         st.lz[h] = (float)a;
         st.uz[h] = (float)c;
-        st.nfree[h] = __float_as_int(val(4));
+        st.nfree[h] = nf;
         a += (double)L.b[i];
         c += (double)L.b[i];
         if (splits && a < 0.0 && c > 0.0) {
@@ -435,13 +454,24 @@ void tl_launch_ibp_box(int grid, const DNet& net, const DState& st, cudaStream_t
     k_ibp_box<<<grid, CB_THREADS, 0, s>>>(net, st);
 }
 
-void tl_launch_ibp(const DNet& net, const DState& st, const TlSeg& seg, const signed char* splits, cudaStream_t s) {
+// Splits of a layer's walks: a layer is one launch, and one with fewer tiles than two per SM (linear layers:
+// 64 at 256 subproblems and 512 rows) leaves most of the chip idle while its blocks walk all their sources. At
+// least 64 taps per split. Without splits 13 conv4 boxes took 1.61 ms, a warp per row 1.53, split 0.60.
+int tl_ibp_splits(const TlSeg& g, int S) {
+    return std::max(1, std::min({152 * 2 / tl_tiles(g, S), g.nch, 16, g.SC * g.kt / 64}));
+}
+
+void tl_launch_ibp(const DNet& net, const DState& st, const TlSegs& segs, int q, const signed char* splits, cudaStream_t s) {
     TlSegs one{};
     one.n = 1;
-    one.s[0] = seg;
+    one.s[0] = segs.s[q];
     one.s[0].first = 0;
-    one.s[0].ks = 1;   // compensated sums are not split
-    k_ibp_tl<<<tl_tiles(seg, net.S), CB_THREADS, tl_ibp_smem(seg), s>>>(net, st, one, splits);
+    one.s[0].ks = tl_ibp_splits(segs.s[q], net.S);
+    one.s[0].part = 0;   // one launch at a time uses the context's scratch
+    one.s[0].ctr = 0;
+    one.part = segs.part;
+    one.ctr = segs.ctr;
+    k_ibp_tl<<<tl_tiles(segs.s[q], net.S) * one.s[0].ks, CB_THREADS, tl_ibp_smem(segs.s[q]), s>>>(net, st, one, splits);
 }
 
 }  // namespace cb
