@@ -24,6 +24,7 @@ constexpr int TL_MAXSEG = 28;       // segments of a launch
 
 struct TlSeg {
     int li, first;          // layer; first block
+    int linear;             // a linear layer's: one position, a subproblem's records neighbours
     int P, Wq;              // positions per subproblem and per line of its grid
     int ch;                 // channels per thread
     int lw, nsub, npt;      // lane warps; subproblems per tile; tiles per subproblem (nsub = 1)
@@ -154,8 +155,9 @@ __device__ __forceinline__ bool tl_unit(const TlSeg& g, const TlTile& t, int l, 
 template <class Op>
 __device__ __forceinline__ void tl_stage(const TlSeg& g, const TlTile& t, int S, int chunk, uint32_t buf, const Op& op) {
     const int c0 = chunk * g.CK, nc = min(g.CK, g.SC - c0), nrec = tl_records(g);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (g.WN == 1) {   // linear: a subproblem's records are neighbours, source channel fastest
+    // (a conv layer's window can be one record as well: its chunks are no power of two, and its source
+    // channels may lie further apart)
+    if (g.linear) {   // a subproblem's records are neighbours, source channel fastest
         for (int i = threadIdx.x; i < g.CK * g.nsub; i += CB_THREADS) {
             const int c = i & (g.CK - 1), sub = i >> (31 - __clz(g.CK));
             if (c < nc && t.s0 + sub < S) op.copy(buf, nrec, c * g.CS + sub, t.s0 + sub, c0 + c);
@@ -163,11 +165,14 @@ __device__ __forceinline__ void tl_stage(const TlSeg& g, const TlTile& t, int S,
     } else {
         const int row = g.row0 + t.p0 / g.Wq * g.step;
         const int n = min(g.WN, (g.rows - row) * g.WX);
-        for (int q = warp; q < nc * g.nsub; q += CB_WARPS) {
+        // a run of n records per (source channel, subproblem), by as many lanes of a warp as it has records
+        const int lg = g.WN >= 32 ? 5 : g.WN > 1 ? 32 - __clz(g.WN - 1) : 0;
+        const int lane = threadIdx.x & ((1 << lg) - 1);
+        for (int q = threadIdx.x >> lg; q < nc * g.nsub; q += CB_THREADS >> lg) {
             const int c = q / g.nsub, sub = q - c * g.nsub;
             if (t.s0 + sub >= S) continue;
             const int src = (c0 + c) * g.cs + row * g.WX, slot = c * g.CS + sub * g.WN;
-            for (int i = lane; i < n; i += 32) op.copy(buf, nrec, slot + i, t.s0 + sub, src + i);
+            for (int i = lane; i < n; i += 1 << lg) op.copy(buf, nrec, slot + i, t.s0 + sub, src + i);
         }
     }
     const int TC = tl_channels(g), lp = 31 - __clz(TC * Op::WB / 16);   // log2 of a weight row's 16-byte pieces

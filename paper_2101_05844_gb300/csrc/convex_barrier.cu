@@ -405,6 +405,7 @@ static int build_tiles(as_ctx* c, const std::vector<std::vector<float>>& Wh) {
             Plan p{};
             TlSeg& g = p.g;
             g.li = k;
+            g.linear = lin;
             g.P = lin ? 1 : L.ho * L.wo;
             g.Wq = lin ? 1 : L.wo;
             g.C = L.co;
@@ -430,6 +431,7 @@ static int build_tiles(as_ctx* c, const std::vector<std::vector<float>>& Wh) {
                 Plan p{};
                 TlSeg& g = p.g;
                 g.li = k;
+                g.linear = lin;
                 g.C = L.ci;
                 g.SC = L.co;
                 g.step = 1;

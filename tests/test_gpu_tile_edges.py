@@ -1,0 +1,120 @@
+"""The tiled walks (csrc/cb_tile.cuh) against the oracle, where their staging can go wrong: batches of a few
+distinct subproblems repeated until the layers take tiles. Copies of a subproblem walk the same taps in the
+same order wherever in a tile they lie, so they have to agree bit for bit; the first of each is compared with
+the oracle, with the tolerances of tests/test_gpu_parity.py."""
+import numpy as np
+import pytest
+
+from oracle import envelope as ev
+from oracle import network as nw
+from paper_2101_05844_gb300 import binding, synth
+from tests.lockstep import check_active_set_step
+from tests.state_helpers import draw_state, hidden_concat, oracle_bounds_f32, split_hidden
+from tests.test_gpu_parity import _draw_sp_state, _install_sp_state
+
+pytestmark = pytest.mark.gpu
+
+DISTINCT = 7   # no divisor of a tile's 32 to 256 subproblems
+
+# Conv layers whose window is one record: a 1x1 kernel on a plane of one position, a kernel that covers its
+# plane (each stride phase of the col pass has one record), a stride that leaves one row of a taller plane
+ONE_RECORD = {
+    "1x1 plane": (synth._convnet((32, 1, 1), [(96, 1, 1, 0), (40, 1, 1, 0)], [24, 3]), 4103),
+    "2x2 to 1x1": (synth._convnet((16, 2, 2), [(24, 2, 2, 0), (20, 1, 1, 0)], [65, 3]), 9101),
+    "2x1 plane": (synth._convnet((20, 2, 1), [(12, 1, 2, 0)], [65, 40, 3]), 8401),
+}
+
+
+def _spread(a, S, axis):
+    """Array a of the distinct subproblems, repeated along `axis` to S."""
+    return np.take(a, np.arange(S) % DISTINCT, axis)
+
+
+def _firsts(a, axis=0):
+    """The distinct subproblems' part of a batch array whose copies are equal bit for bit."""
+    first = np.take(a, np.arange(DISTINCT), axis)
+    np.testing.assert_array_equal(a, _spread(first, a.shape[axis], axis))
+    return first
+
+
+@pytest.mark.parametrize("cap", [3, 5])
+@pytest.mark.parametrize("name", list(ONE_RECORD))
+def test_windows_of_one_record(name, cap):
+    import torch
+    layers, S = ONE_RECORD[name]
+    net = synth.make_net(layers, 3)
+    work = S * sum(L["W"].size * (L["out_shape"][1] * L["out_shape"][2] if L["kind"] == "conv" else 1) for L in net[:-1])
+    assert work >= 3e7, "the batch must be large enough for tiles"
+    c, lo, hi = synth.make_boxes(net[0]["n_in"], DISTINCT, 0.1, 4)
+    C = synth.properties_runner_up(synth.forward(net, c))
+    dense = nw.dense_layers(net)
+    prob = dict(net=net, lo=lo, hi=hi, C=C)
+    Ps = nw.problems(prob, dense=dense)
+    rep = lambda a, axis=0: _spread(a, S, axis)  # noqa: E731
+
+    # interval propagation
+    kw = dict(bigm_iters=5, as_iters=40, omega=3, max_cuts=cap)
+    opt = binding.default_options(graph_chunk=0, **kw)
+    big = binding.Context(net, rep(lo), rep(hi), rep(C), options=opt)
+    hidden = lambda w, dt=np.float32: big.get_state(w, dt).reshape(S, -1)  # noqa: E731
+    lh, uh = _firsts(hidden(binding.ST_LHAT)), _firsts(hidden(binding.ST_UHAT))
+    for s, P in enumerate(Ps):
+        rl, ru = hidden_concat(P.lhat), hidden_concat(P.uhat)
+        assert (lh[s] <= rl + 1e-9 * (1 + np.abs(rl))).all() and (uh[s] >= ru - 1e-9 * (1 + np.abs(ru))).all()
+        assert (np.abs(lh[s] - rl) <= 4e-6 * (1 + np.abs(rl))).all()
+        assert (np.abs(uh[s] - ru) <= 4e-6 * (1 + np.abs(ru))).all()
+
+    # an Active Set iteration from a drawn state that adds slot 2, and the gradient there
+    lh, uh = oracle_bounds_f32(Ps)
+    Ps = nw.problems(prob, bounds=[(split_hidden(lh[s].astype(np.float64), Ps[0].widths)[1:],
+                                    split_hidden(uh[s].astype(np.float64), Ps[0].widths)[1:])
+                                   for s in range(DISTINCT)], dense=dense)
+    big.reset(rep(lo), rep(hi), rep(C), rep(lh), rep(uh))
+    few = binding.Context(net, lo, hi, C, lh, uh, options=opt)
+    solvers = draw_state(Ps, few, kw, it=8, nslots=2, seed=31)
+    shapes = {binding.ST_ALPHA: ((DISTINCT, -1), 0), binding.ST_BETA0: ((DISTINCT, -1), 0),
+              binding.ST_BETA1: ((DISTINCT, -1), 0), binding.ST_ADAM: ((6, DISTINCT, -1), 1),
+              binding.ST_SLOT_ADAM: ((2, DISTINCT, -1), 1), binding.ST_XSNAP: ((DISTINCT, -1), 0),
+              binding.ST_ZSNAP: ((DISTINCT, -1), 0), binding.ST_SLOT_BETA: ((DISTINCT, -1), 0)}
+    big.set_state(binding.ST_ITER, few.get_state(binding.ST_ITER, np.int32))
+    for w, (shape, axis) in shapes.items():
+        dt = np.uint8 if w in (binding.ST_XSNAP, binding.ST_ZSNAP) else np.float32
+        big.set_state(w, rep(few.get_state(w, dt).reshape(shape), axis))
+    n0 = lo.shape[1]
+    dlo, dhi = (torch.zeros((S, n0), device="cuda") for _ in range(2))
+    big.backward(np.ones(S), None, None, dlo, dhi)
+    dlo, dhi = _firsts(dlo.cpu().numpy()), _firsts(dhi.cpu().numpy())
+    bound = _firsts(big.bound(64))
+    for s, sv in enumerate(solvers):
+        g = ev.envelope_gradient(sv.P, sv.st)
+        assert bound[s] == pytest.approx(g["value"], abs=1e-4, rel=1e-5)
+        for got, ref in ((dlo[s], g["dlo0"]), (dhi[s], g["dhi0"])):
+            np.testing.assert_allclose(got, ref, rtol=1e-4, atol=1e-4 * np.abs(ref).max())
+    big.as_step(1)
+    al, b0, b1 = (_firsts(hidden(w)) for w in (binding.ST_ALPHA, binding.ST_BETA0, binding.ST_BETA1))
+    sb = _firsts(hidden(binding.ST_SLOT_BETA)).reshape(DISTINCT, big.cap, -1)
+    xstar = _firsts(hidden(binding.ST_XSTAR))
+    for s, sv in enumerate(solvers):
+        check_active_set_step(sv, dict(alpha=al[s], beta0=b0[s], beta1=b1[s], slots=sb[s], xstar=xstar[s]))
+
+    # a Saddle Point iteration from a drawn iterate
+    sps, st = _draw_sp_state(Ps, 50, 4)
+    _install_sp_state(big, dict(x=rep(st["x"]), z=rep(st["z"]), stats=rep(st["stats"], 1), caps=rep(st["caps"], 1),
+                                alpha=rep(st["alpha"])), 4)
+    value = _firsts(big.bound())
+    big.sp_step(1)
+    sel, x, z = _firsts(hidden(binding.ST_SP_SEL, np.uint8)), _firsts(hidden(binding.ST_SP_X)), _firsts(hidden(binding.ST_SP_Z))
+    al = _firsts(hidden(binding.ST_ALPHA))
+    stats = _firsts(big.get_state(binding.ST_SP_STATS).reshape(4, S, -1), 1)
+    tol = dict(rtol=1e-5, atol=1e-6)
+    for s, sp in enumerate(sps):
+        assert value[s] == pytest.approx(sp.evaluate()[0], abs=1e-5, rel=1e-5)
+        sp.step(1)
+        np.testing.assert_array_equal(sel[s], hidden_concat(sp.last_sel).astype(np.uint8))
+        np.testing.assert_allclose(x[s], np.concatenate(sp.x), **tol)
+        np.testing.assert_allclose(z[s], hidden_concat(sp.z), **tol)
+        np.testing.assert_allclose(al[s], hidden_concat(sp.alpha), **tol)
+        for q, ref in enumerate((sp.Sb, sp.G, sp.C)):
+            np.testing.assert_allclose(stats[q, s, n0:], hidden_concat(ref), **tol)
+        np.testing.assert_allclose(stats[3, s, :-big.widths[-1]],
+                                   np.concatenate([sp.Pst[k] for k in range(1, sp.P.n)]), **tol)
