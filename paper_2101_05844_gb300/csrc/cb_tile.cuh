@@ -21,6 +21,10 @@
 namespace cb {
 
 constexpr int TL_MAXSEG = 28;       // segments of a launch
+// Dynamic shared memory a tiled kernel may ask for (two blocks per SM). The limit that a kernel is given belongs
+// to the kernel, not to a context: it is this value for every context, never one context's own need, which would
+// have the launches of another context with larger tiles refused.
+constexpr int TL_SMEM_MAX = 100 * 1024;
 
 struct TlSeg {
     int li, first;          // layer; first block
@@ -312,9 +316,9 @@ __device__ __forceinline__ int tl_col_neuron(const DLayer& L, const TlSeg& g, in
 }
 
 // Launches (tile_as.cu). tl_weights fills a segment's weights from its layer's; tl_as_prepare allows
-// the passes their shared memory; seq: the col pass's sums in the lane teams' order.
+// the passes TL_SMEM_MAX; seq: the col pass's sums in the lane teams' order.
 void tl_weights(const DLayer& L, bool col, const TlSeg& g, float* w, float2* wpm, cudaStream_t s);
-cudaError_t tl_as_prepare(int smem_col, int smem_row);
+cudaError_t tl_as_prepare();
 void tl_launch_colA(bool seq, int blocks, int smem, const DNet& net, const DState& st, const DSched& sc, const TlSegs& t,
                     int mode, cudaStream_t s);
 void tl_launch_rowB(int blocks, int smem, const DNet& net, const DState& st, const DSched& sc, const TlSegs& t,
@@ -322,7 +326,7 @@ void tl_launch_rowB(int blocks, int smem, const DNet& net, const DState& st, con
 // Interval propagation (tile_sp.cu): the input box's records, then a row segment per hidden layer.
 int tl_ibp_smem(const TlSeg& g);
 int tl_ibp_splits(const TlSeg& g, int S);
-cudaError_t tl_sp_prepare(int smem_ibp, int smem_row, int smem_col);
+cudaError_t tl_sp_prepare();
 void tl_launch_ibp_box(int grid, const DNet& net, const DState& st, cudaStream_t s);
 void tl_launch_ibp(const DNet& net, const DState& st, const TlSegs& segs, int q, const signed char* splits, cudaStream_t s);
 // Saddle Point (tile_sp.cu): its passes, the col pass's work by `what` (0: phase C and the next phase A, 1:

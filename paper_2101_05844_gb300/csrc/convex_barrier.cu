@@ -363,7 +363,9 @@ static bool tile_shape(TlSeg& g, int S, bool linear, int lines, int span, int rb
         } else {
             while (t.CK < t.SC && t.CK < 64 && fits(t.CK + 1)) ++t.CK;
         }
-        if (tl_smem(t, rb, 8, eb, 0) > 100 * 1024) continue;
+        // (the bound holds for every kernel on these tiles: their records and weights are no larger, and
+        // none stages more sums per unit than a row pass with every slot in use)
+        if (tl_smem(t, rb, 8, eb, 1 + CB_MAXCUT) > TL_SMEM_MAX) continue;
         const double cost = (double)tl_tiles(t, S) * t.SC *
                             (t.kt * 24.0 * t.ch + t.nsub * t.WN * (rb / 32.0) + t.kt * TC * 8 / 32.0);
         if (best < 0 || cost < best) {
@@ -563,14 +565,12 @@ static int build_tiles(as_ctx* c, const std::vector<std::vector<float>>& Wh) {
         c->tlB.part = c->tlA.part;   // the passes of a context run one after the other
         c->tlB.ctr = c->tlA.ctr;
     }
-    CUDA_TRY(c, tl_as_prepare(c->smemLA, c->smemLB));
+    CUDA_TRY(c, tl_as_prepare());
     c->ibp_tiles = c->tlB.n == n - 1;
-    int ibp = 0;
-    for (int q = 0; q < c->tlB.n; ++q) ibp = std::max(ibp, tl_ibp_smem(c->tlB.s[q]));
     c->sp_tiles = c->ibp_tiles && (int)std::count(c->tl_col, c->tl_col + n, true) == n;
     for (int q = 0; q < c->tlB.n; ++q) c->smemSB = std::max(c->smemSB, tl_sp_row_smem(c->tlB.s[q]));
     for (int q = 0; q < c->tlA.n; ++q) c->smemSA = std::max(c->smemSA, tl_sp_col_smem(c->tlA.s[q]));
-    CUDA_TRY(c, tl_sp_prepare(ibp, c->smemSB, c->smemSA));
+    CUDA_TRY(c, tl_sp_prepare());
     return AS_OK;
 }
 

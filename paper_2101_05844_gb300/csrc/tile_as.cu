@@ -504,12 +504,12 @@ void tl_weights(const DLayer& L, bool col, const TlSeg& g, float* w, float2* wpm
     k_tl_weights<<<grid, CB_THREADS, 0, s>>>(L, col, g.py, g.px, g.SC * g.kt, g.C, CP, w, wpm);
 }
 
-cudaError_t tl_as_prepare(int smem_col, int smem_row) {
-    cudaError_t e = cudaFuncSetAttribute(k_as_colA_tl<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_col);
+cudaError_t tl_as_prepare() {
+    cudaError_t e = cudaFuncSetAttribute(k_as_colA_tl<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, TL_SMEM_MAX);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_as_colA_tl<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_col);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_sp_convert_tl, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_col);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_as_rowB_tl, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_row);
+        e = cudaFuncSetAttribute(k_as_colA_tl<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, TL_SMEM_MAX);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_sp_convert_tl, cudaFuncAttributeMaxDynamicSharedMemorySize, TL_SMEM_MAX);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_as_rowB_tl, cudaFuncAttributeMaxDynamicSharedMemorySize, TL_SMEM_MAX);
     return e;
 }
 

@@ -435,18 +435,18 @@ void tl_launch_spi_row(int blocks, int smem, const DNet& net, const DState& st, 
 }
 int tl_ibp_smem(const TlSeg& g) { return tl_smem(g, 8, 4, 0, 5); }
 
-cudaError_t tl_sp_prepare(int smem_ibp, int smem_row, int smem_col) {
+cudaError_t tl_sp_prepare() {
     cudaError_t e = cudaSuccess;
-    auto allow = [&](const void* k, int bytes) {
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    auto allow = [&](const void* k) {
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, TL_SMEM_MAX);
     };
-    allow((const void*)k_ibp_tl, smem_ibp);
-    allow((const void*)k_sp_rowB_tl, smem_row);
-    allow((const void*)k_spi_row_tl, smem_row);
-    allow((const void*)k_sp_col_tl<SP_PHASE_CA>, smem_col);
-    allow((const void*)k_sp_col_tl<SP_PHASE_A>, smem_col);
-    allow((const void*)k_sp_col_tl<SP_START>, smem_col);
-    allow((const void*)k_sp_col_tl<SP_INIT>, smem_col);
+    allow((const void*)k_ibp_tl);
+    allow((const void*)k_sp_rowB_tl);
+    allow((const void*)k_spi_row_tl);
+    allow((const void*)k_sp_col_tl<SP_PHASE_CA>);
+    allow((const void*)k_sp_col_tl<SP_PHASE_A>);
+    allow((const void*)k_sp_col_tl<SP_START>);
+    allow((const void*)k_sp_col_tl<SP_INIT>);
     return e;
 }
 
