@@ -155,6 +155,13 @@ __device__ __forceinline__ bool tl_unit(const TlSeg& g, const TlTile& t, int l, 
     return sub < g.nsub && s < S && p < g.P;
 }
 
+// What a walk's op may leave as it is here: taken() hears of the taps after every four of them (a chunk's last
+// ones singly), or after each with singly().
+struct TlOp {
+    __device__ __forceinline__ bool singly() const { return false; }
+    __device__ __forceinline__ void taken(int) {}
+};
+
 // One chunk into a buffer: op copies record `src` of subproblem s into slot `slot`.
 template <class Op>
 __device__ __forceinline__ void tl_stage(const TlSeg& g, const TlTile& t, int S, int chunk, uint32_t buf, const Op& op) {
@@ -217,14 +224,19 @@ __device__ __forceinline__ void tl_walk(const TlSeg& g, const TlTile& t, int S, 
                 __syncthreads();
             }
             int k = 0;
-            for (; k + 4 <= nk; k += 4) {
+            const int nk4 = op.singly() ? 0 : nk;
+            for (; k + 4 <= nk4; k += 4) {
                 const int4 o = *reinterpret_cast<const int4*>(ko + k);
                 op.step(rec, ex, nrec, t.win + o.x, w + (k + 0) * TC * Op::WB);
                 op.step(rec, ex, nrec, t.win + o.y, w + (k + 1) * TC * Op::WB);
                 op.step(rec, ex, nrec, t.win + o.z, w + (k + 2) * TC * Op::WB);
                 op.step(rec, ex, nrec, t.win + o.w, w + (k + 3) * TC * Op::WB);
+                op.taken(4);
             }
-            for (; k < nk; ++k) op.step(rec, ex, nrec, t.win + ko[k], w + k * TC * Op::WB);
+            for (; k < nk; ++k) {
+                op.step(rec, ex, nrec, t.win + ko[k], w + k * TC * Op::WB);
+                op.taken(1);
+            }
             __syncthreads();
         }
         op.end(sweep);

@@ -110,4 +110,21 @@ struct CompSum {
     __device__ __forceinline__ double warp_total() const { return warp_sum((double)s + (double)c); }
 };
 
+// The sum of many such pairs, beyond float64's accuracy in three float32 words: a pair's two words are added by
+// TwoSum to the first and second, the first's rounding errors to the second, the second's to the third.
+struct CompTotal {
+    float s = 0.f, c = 0.f, d = 0.f;
+    static __device__ __forceinline__ float two_sum(float& a, float b) {   // a becomes a + b; returns its error
+        const float t = __fadd_rn(a, b), z = __fsub_rn(t, a);
+        const float e = __fadd_rn(__fsub_rn(a, __fsub_rn(t, z)), __fsub_rn(b, z));
+        a = t;
+        return e;
+    }
+    __device__ __forceinline__ void add(const CompSum& q) {
+        const float e = two_sum(s, q.s), ec = two_sum(c, q.c), ee = two_sum(c, e);
+        d = __fadd_rn(d, __fadd_rn(ec, ee));
+    }
+    __device__ __forceinline__ double total() const { return (double)s + ((double)c + (double)d); }
+};
+
 }  // namespace cb

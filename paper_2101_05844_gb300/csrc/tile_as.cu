@@ -47,7 +47,7 @@ __global__ void k_tl_weights(DLayer L, int col, int py, int px, int rows, int C,
 // ---------------------------------------------------------------- col pass
 // Output records {rp, bz_b}: plane q holds entries 4q .. 4q + 3; only the 1 + NS entries in use are staged.
 template <int NS>
-struct ColRecords {
+struct ColRecords : TlOp {
     static constexpr int E = 1 + NS, RB = tl_arec_bytes(E), EB = 0;
     const float4* src;      // the layer's records of subproblem 0
     size_t ss;              // float4 per subproblem
@@ -359,7 +359,7 @@ __global__ void __launch_bounds__(CB_THREADS, 2) k_sp_convert_tl(DNet net, DStat
 // spread into one pair {x* p_b, x* q_b} per slot when a chunk has arrived: picked per tap, the bits cost
 // as many instructions as the products (conv4 net, 64 boxes, five slots: 526 M instructions a pass).
 template <int NS, int CH>
-struct RowOp {
+struct RowOp : TlOp {
     static constexpr int RB = 8, EB = 8 * NS, WB = NS ? 8 : 4, SWEEPS = 1;
     const float2* src;
     size_t ss;              // records per subproblem

@@ -7,18 +7,26 @@ namespace cb {
 
 // ---------------------------------------------------------------- interval propagation
 // Interval propagation (App. E) of one hidden layer on tiles: lhat = W+ l + W- u + b, uhat = W+ u + W- l + b
-// by compensated float32 sums (CompSum: float64 accuracy), from records {l, u} of the layer's inputs
-// kept in the first Saddle Point input plane. A warp per row (k_ibp) reads every weight and bound of a
-// row from L1 for that row alone: 26.6 ms for 256 conv4 boxes, where the sums' 20 operations per tap take
-// about 1.6 ms at the float32 rate. On tiles 4.5 ms, and 4.0 with the layers of few tiles split over their
-// sources (tl_ibp_splits).
+// by compensated float32 sums, from records {l, u} of the layer's inputs kept in the first Saddle Point input
+// plane. A warp per row (k_ibp) reads every weight and bound of a row from L1 for that row alone: 26.6 ms for
+// 256 conv4 boxes, where the sums' 20 operations per tap take about 1.6 ms at the float32 rate. On tiles 4.7
+// ms (the layers of few tiles split over their sources, tl_ibp_splits).
+//
+// Accuracy: a pair (CompSum) loses about k 2^-48 over k terms, so one pair over a whole row is worse than the
+// warp's 32 pairs that meet in float64 (rms over rows of 576 terms 1.1e-15 against 3.4e-16 of the terms'
+// magnitudes). A thread's pair therefore ends where a lane's would, after a 32nd of the row, and goes into a
+// three-word total (CompTotal): no larger error than the warp's at any of 27 to 8192 terms. That costs 20
+// operations per 32nd of a row (4.0 -> 4.7 ms); adding into float64 instead would take about 6 ms on its narrow
+// pipe alone.
 template <int CH>
-struct IbpOp {
+struct IbpOp : TlOp {
     static constexpr int RB = 8, EB = 0, WB = 4, SWEEPS = 1;
     const float4* src;      // the layer's input records of subproblem 0
     size_t ss;              // records per subproblem
     CompSum a[CH], c[CH];
+    CompTotal ta[CH], tc[CH];
     int nf[CH];
+    int part, room;         // taps of a pair; taps the present one has left
     __device__ __forceinline__ void copy(uint32_t buf, int, int slot, int s, int i) const {
         tl_copy<8>(buf + slot * 8, src + (size_t)s * ss + i);
     }
@@ -26,6 +34,15 @@ struct IbpOp {
     __device__ __forceinline__ void begin(int) {
 #pragma unroll
         for (int k = 0; k < CH; ++k) nf[k] = 0;
+        room = part;
+    }
+    __device__ __forceinline__ bool singly() const { return part < 4; }
+    __device__ __forceinline__ void taken(int n) {
+        room -= n;
+        if (room < (part < 4 ? 1 : 4)) {
+            end(0);
+            room = part;
+        }
     }
     __device__ __forceinline__ void step(const char* rec, const char*, int, int slot, const char* w) {
         const float2 r = *reinterpret_cast<const float2*>(rec + slot * 8);
@@ -43,7 +60,14 @@ struct IbpOp {
             }
         }
     }
-    __device__ __forceinline__ void end(int) {}
+    __device__ __forceinline__ void end(int) {   // the pairs into the totals
+#pragma unroll
+        for (int k = 0; k < CH; ++k) {
+            ta[k].add(a[k]);
+            tc[k].add(c[k]);
+            a[k] = c[k] = CompSum{};
+        }
+    }
 };
 
 // Layer k's records {l, u} of its inputs from the input box (k = 0; later layers' are written by the
@@ -70,19 +94,22 @@ __device__ __forceinline__ void ibp_tile(const DNet& net, const DState& st, cons
         IbpOp<CH> op;
         op.src = slot_rec_plane(net, st, L, 0);
         op.ss = net.XT;
+        // a pair takes the terms that a lane of the warp walk takes (conv: rows of kernel columns)
+        op.part = max(g.SC * g.kt / 32, L.kw);
         tl_walk(g, t, net.S, smem, op);
         float v[CH][5];
 #pragma unroll
-        for (int k = 0; k < CH; ++k) {
-            v[k][0] = op.a[k].s;
-            v[k][1] = op.a[k].c;
-            v[k][2] = op.c[k].s;
-            v[k][3] = op.c[k].c;
+        for (int k = 0; k < CH; ++k) {   // the float64 sums as words
+            const double a = op.ta[k].total(), c = op.tc[k].total();
+            v[k][0] = __int_as_float(__double2loint(a));
+            v[k][1] = __int_as_float(__double2hiint(a));
+            v[k][2] = __int_as_float(__double2loint(c));
+            v[k][3] = __int_as_float(__double2hiint(c));
             v[k][4] = __int_as_float(op.nf[k]);
         }
         tl_put<5, CH>(g, t, sums, v);
     }
-    // the splits' pairs of a row are added in float64 by the block that arrives last
+    // the splits' sums of a row are added in float64 by the block that arrives last
     if (g.ks > 1 && !tl_arrive<5>(segs, g, t, sums)) return;
     __syncthreads();
     const int TC = tl_channels(g), row = tl_lanes(g) + 1;
@@ -95,18 +122,18 @@ __device__ __forceinline__ void ibp_tile(const DNet& net, const DState& st, cons
         double a = 0.0, c = 0.0;
         int nf = 0;
         if (g.ks == 1) {
-            auto val = [&](int e) { return sums[e * TC * row + at]; };
-            a = (double)val(0) + (double)val(1);
-            c = (double)val(2) + (double)val(3);
-            nf = __float_as_int(val(4));
+            auto val = [&](int e) { return __float_as_int(sums[e * TC * row + at]); };
+            a = __hiloint2double(val(1), val(0));
+            c = __hiloint2double(val(3), val(2));
+            nf = val(4);
         } else {
 #pragma unroll 4
             for (int q = 0; q < g.ks; ++q) {
                 const float* v = part + q * tl_split(g, 5) + at;
-                auto val = [&](int e) { return __ldcg(v + e * TC * row); };
-                a += (double)val(0) + (double)val(1);
-                c += (double)val(2) + (double)val(3);
-                nf += __float_as_int(val(4));
+                auto val = [&](int e) { return __float_as_int(__ldcg(v + e * TC * row)); };
+                a += __hiloint2double(val(1), val(0));
+                c += __hiloint2double(val(3), val(2));
+                nf += val(4);
             }
         }
         const size_t h = (size_t)s * net.NH + L.h_out + i;
@@ -145,7 +172,7 @@ __global__ void __launch_bounds__(CB_THREADS, 2) k_ibp_tl(DNet net, DState st, c
 // threshold of the tap's sign, a few selects per tap and channel; a record {x, tau+, tau-, l, u} is staged
 // once per tile where the lane teams loaded 16 bytes per unit and tap. Bound by issue.
 template <int CH>
-struct SpRowOp {
+struct SpRowOp : TlOp {
     static constexpr int RB = 20, EB = 0, WB = 4, SWEEPS = 1;
     const float4* src;      // the layer's records of subproblem 0: {x, tau+, l, u}, and xpos on {x, tau-, u, l}
     size_t ss;
@@ -246,7 +273,7 @@ __global__ void __launch_bounds__(CB_THREADS, 2) k_sp_rowB_tl(DNet net, DState s
 
 // Phase C fused with the next phase A (k_sp_colCA_t): the output records {alpha, beta_bar on beta_1, beta_bar on I*, z}.
 template <int CH>
-struct SpColOp {
+struct SpColOp : TlOp {
     static constexpr int RB = 16, EB = 0, WB = 4, SWEEPS = 1;
     const float4* src;
     size_t ss;
@@ -280,7 +307,7 @@ struct SpColOp {
 // W x or W^T y of the first entries of float4 records: phase A alone (alpha), the primal initialisation's
 // products (x; alpha* - beta_1*).
 template <int CH>
-struct DotOp {
+struct DotOp : TlOp {
     static constexpr int RB = 4, EB = 0, WB = 4, SWEEPS = 1;
     const float4* src;
     size_t ss;
