@@ -234,7 +234,9 @@ long long as_launch_count(as_ctx* ctx);
 #define AS_K_COUNT 15
 
 /* With as_options.profile set: total device time (CUDA events on the context's stream) and
- * launch count of one kernel over the context's life so far. Synchronises the stream. */
+ * launch count of one kernel over the context's life so far. A col or row pass counts once per
+ * iteration, also where its layers are shared between two kernels (as_launch_count counts both).
+ * Synchronises the stream. */
 int as_kernel_times(as_ctx* ctx, int kernel, double* total_ms, long long* launches);
 
 void as_destroy(as_ctx* ctx);

@@ -849,6 +849,15 @@ static cudaEvent_t prof_event(as_ctx* c) {
         }                                                          \
         (c)->launches++;                                           \
     } while (0)
+// A pass over all layers that may take two kernels, `first` for the layers that qualify for it (has1) and
+// `second` for the rest (has2): timed and counted as one launch of the pass, since as_kernel_times' counts stand
+// for iterations; as_launch_count has both.
+#define LAUNCH_PASS(c, s, id, has1, first, has2, second)           \
+    do {                                                           \
+        const bool a_ = (has1), b_ = (has2);                       \
+        LAUNCH(c, s, id, if (a_) first; if (b_) second);           \
+        if (a_ && b_) (c)->launches++;                             \
+    } while (0)
 
 // Box, property rows, intermediate bounds, splits and caps of a batch; zeroes the duals.
 static int load_batch(as_ctx* c, const float* x_lo, const float* x_hi, const float* C, const float* lhat,
@@ -1191,12 +1200,9 @@ static void launch_after(as_ctx* c, void (*k)(P...), int grid, int threads, cuda
 // The float32 col pass: the tiled layers, then the lane teams' share; seq: the tiles' sums in the lane
 // teams' order.
 static void launch_colA(as_ctx* c, cudaStream_t s, int mode, bool seq) {
-    if (c->blocksLA)
-        LAUNCH(c, s, CB_K_AS_COLA,
-               tl_launch_colA(seq, c->blocksLA, c->smemLA, c->net, c->st, c->sc, c->tlA, mode, s));
-    if (c->blocksTAr)
-        LAUNCH(c, s, CB_K_AS_COLA,
-               launch_after(c, k_as_colA_t<false>, c->blocksTAr, CB_THREADS, s, c->net, c->st, c->sc, c->tAr, mode));
+    LAUNCH_PASS(c, s, CB_K_AS_COLA, c->blocksLA,
+                tl_launch_colA(seq, c->blocksLA, c->smemLA, c->net, c->st, c->sc, c->tlA, mode, s), c->blocksTAr,
+                launch_after(c, k_as_colA_t<false>, c->blocksTAr, CB_THREADS, s, c->net, c->st, c->sc, c->tAr, mode));
 }
 
 static int launch_as_iter(as_ctx* c, cudaStream_t s) {
@@ -1206,11 +1212,9 @@ static int launch_as_iter(as_ctx* c, cudaStream_t s) {
     if (c->net.ball) LAUNCH(c, s, CB_K_BALL_X0, (k_ball_x0<<<c->net.S, CB_BALL_THREADS, 0, s>>>(c->net, c->st)));
     if (c->opt.track_best)
         LAUNCH(c, s, CB_K_REDUCE, launch_after(c, k_reduce, c->net.S, CB_THREADS, s, c->net, c->st, 64, (double*)nullptr, 1));
-    if (c->blocksLB)
-        LAUNCH(c, s, CB_K_AS_ROWB, tl_launch_rowB(c->blocksLB, c->smemLB, c->net, c->st, c->sc, c->tlB, s));
-    if (c->blocksTBr)
-        LAUNCH(c, s, CB_K_AS_ROWB,
-               launch_after(c, k_as_rowB_t<false>, c->blocksTBr, CB_THREADS, s, c->net, c->st, c->sc, c->tBr));
+    LAUNCH_PASS(c, s, CB_K_AS_ROWB, c->blocksLB,
+                tl_launch_rowB(c->blocksLB, c->smemLB, c->net, c->st, c->sc, c->tlB, s), c->blocksTBr,
+                launch_after(c, k_as_rowB_t<false>, c->blocksTBr, CB_THREADS, s, c->net, c->st, c->sc, c->tBr));
     LAUNCH(c, s, CB_K_COUNTER, launch_after(c, k_advance, 1, 32, s, c->st, c->sc, 0));
     return check_launch(c, "Active Set iteration");
 }

@@ -84,3 +84,23 @@ def test_branch_and_bound_with_its_default_options():
     vals = synth.forward(net, x) @ C[0]
     assert res["bounded"] >= 2
     assert np.isfinite(res["lower"]) and res["lower"] <= vals.min() + 1e-5 and res["lower"] <= res["upper"]
+
+
+@pytest.mark.parametrize("name,S,sparse,precision", [("mlp_300_200_200_3", 600, True, 32), ("mlp_32_24_22_18_3", 6, False, 16)])
+def test_a_pass_of_two_kernels_counts_once_per_iteration(name, S, sparse, precision):
+    """Kernel times of a net whose layers are shared between two kernels: tiles and lane teams (a layer of mostly
+    zero weights), or four neurons and one neuron a thread (offsets of some layers only are multiples of four)."""
+    net, lo, hi, C = _problem(name, S)
+    if sparse:
+        W = net[1]["W"]
+        W[np.random.default_rng(3).random(W.shape) < 0.9] = 0
+    ctx = binding.Context(net, lo, hi, C, options=binding.default_options(profile=1, max_cuts=2, bigm_iters=3, as_iters=20,
+                                                                         precision=precision))
+    t0, l0 = ctx.kernel_times(), ctx.launch_count()
+    ctx.as_step(8)
+    t1, launches = ctx.kernel_times(), ctx.launch_count() - l0
+    count = {k: t1[k][1] - t0[k][1] for k in t1}
+    assert count["as_colA"] == count["as_rowB"] == count["counter"] == 8
+    assert t1["as_colA"][0] > 0 and t1["as_rowB"][0] > 0
+    # two kernels a pass, and the other kernels one launch per count
+    assert launches == sum(count.values()) + 2 * 8
