@@ -1006,7 +1006,8 @@ static int time_iters(as_ctx* c, int reps, float* ms) {
 }
 
 // as_options.autotune: the team-size targets of the col pass, then of the row pass, each the
-// fastest of a doubling sequence on this context's own net and batch. The caller reloads the
+// fastest of a doubling sequence on this context's own net and batch. A pass whose layers are all on
+// tiles reads no target: its times would be noise, and it keeps the default. The caller reloads the
 // batch afterwards (the timing iterations move the duals).
 static int autotune_teams(as_ctx* c) {
     static const long long cand[] = {5000, 10000, 20000, 40000, 80000, 160000, 320000};
@@ -1015,6 +1016,7 @@ static int autotune_teams(as_ctx* c) {
     for (int pass = 0; pass < 2; ++pass) {
         // a target pinned by CB_TEAM_TARGET_COL / CB_TEAM_TARGET_ROW is not tuned
         if (getenv(pass ? "CB_TEAM_TARGET_ROW" : "CB_TEAM_TARGET_COL")) continue;
+        if (!(pass ? c->blocksTBr : c->blocksTAr)) continue;
         long long best = pass ? c->team_row : c->team_col;
         float best_ms = 0.f;
         for (long long t : cand) {
@@ -1127,7 +1129,7 @@ static int init_impl(as_ctx* c, const as_net* net, int S, const float* x_lo, con
     TRY(build_tables(c));
     if (c->opt.precision == 16) TRY(build_bf16(c, Wh));
     TRY(load_batch(c, x_lo, x_hi, C, lhat, uhat, splits, caps, true));
-    if (c->opt.autotune && c->opt.precision == 32) {
+    if (c->opt.autotune && c->opt.precision == 32 && (c->blocksTAr || c->blocksTBr)) {
         TRY(autotune_teams(c));
         TRY(load_batch(c, x_lo, x_hi, C, lhat, uhat, splits, caps, false));   // back to zero duals
     }

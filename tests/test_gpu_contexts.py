@@ -104,3 +104,17 @@ def test_a_pass_of_two_kernels_counts_once_per_iteration(name, S, sparse, precis
     assert t1["as_colA"][0] > 0 and t1["as_rowB"][0] > 0
     # two kernels a pass, and the other kernels one launch per count
     assert launches == sum(count.values()) + 2 * 8
+
+
+def test_autotune_leaves_passes_on_tiles_alone():
+    """Team-size targets mean nothing to a pass whose layers are all on tiles: none is timed there, and the
+    default stays; a net with a layer of mostly zero weights has targets to time."""
+    net, lo, hi, C = _problem("mlp_300_200_200_3", 600)
+    make = lambda tune: binding.Context(net, lo, hi, C, options=binding.default_options(  # noqa: E731
+        bigm_iters=3, as_iters=20, autotune=tune))
+    plain, tuned = make(0), make(1)
+    assert tuned.team_targets() == plain.team_targets() == (40000, 40000)
+    assert tuned.launch_count() <= 2 * plain.launch_count()   # set-up only, no timed iterations
+    W = net[1]["W"]
+    W[np.random.default_rng(3).random(W.shape) < 0.9] = 0
+    assert make(1).launch_count() > 2 * plain.launch_count()
