@@ -5,6 +5,7 @@ the oracle, with the tolerances of tests/test_gpu_parity.py."""
 import numpy as np
 import pytest
 
+from oracle import dual as du
 from oracle import envelope as ev
 from oracle import network as nw
 from paper_2101_05844_gb300 import binding, synth
@@ -40,8 +41,28 @@ def _firsts(a, axis=0):
 @pytest.mark.parametrize("cap", [3, 5])
 @pytest.mark.parametrize("name", list(ONE_RECORD))
 def test_windows_of_one_record(name, cap):
+    _check_against_oracle(*ONE_RECORD[name], cap, it=8, nslots=2)
+
+
+# Planes larger and smaller than a tile, stride phases of unequal size, channels that are no multiple of a thread's,
+# stride 3, narrow and odd linear layers
+GENERAL = {
+    "odd planes": (synth._convnet((3, 13, 11), [(5, 3, 1, 1), (9, 3, 2, 1), (12, 4, 3, 2)], [33, 3]), 701),
+    "tall kernel": (synth._convnet((2, 9, 40), [(10, 5, 2, 0)], [17, 2]), 900),
+    "linear": (synth._mlp([300, 65, 7, 130, 4]), 1537),
+}
+
+
+@pytest.mark.parametrize("cap,it,nslots", [(3, 8, 2), (8, 14, 6)])
+@pytest.mark.parametrize("name", list(GENERAL))
+def test_tiles_against_the_oracle(name, cap, it, nslots):
+    _check_against_oracle(*GENERAL[name], cap, it, nslots)
+
+
+def _check_against_oracle(layers, S, cap, it, nslots):
+    """Interval bounds, the gradient and an iteration of Active Set (global iteration `it`, which adds slot nslots),
+    and an iteration of Saddle Point, from drawn states."""
     import torch
-    layers, S = ONE_RECORD[name]
     net = synth.make_net(layers, 3)
     work = S * sum(L["W"].size * (L["out_shape"][1] * L["out_shape"][2] if L["kind"] == "conv" else 1) for L in net[:-1])
     assert work >= 3e7, "the batch must be large enough for tiles"
@@ -64,14 +85,14 @@ def test_windows_of_one_record(name, cap):
         assert (np.abs(lh[s] - rl) <= 4e-6 * (1 + np.abs(rl))).all()
         assert (np.abs(uh[s] - ru) <= 4e-6 * (1 + np.abs(ru))).all()
 
-    # an Active Set iteration from a drawn state that adds slot 2, and the gradient there
+    # an Active Set iteration from a drawn state, and the gradient there
     lh, uh = oracle_bounds_f32(Ps)
     Ps = nw.problems(prob, bounds=[(split_hidden(lh[s].astype(np.float64), Ps[0].widths)[1:],
                                     split_hidden(uh[s].astype(np.float64), Ps[0].widths)[1:])
                                    for s in range(DISTINCT)], dense=dense)
     big.reset(rep(lo), rep(hi), rep(C), rep(lh), rep(uh))
     few = binding.Context(net, lo, hi, C, lh, uh, options=opt)
-    solvers = draw_state(Ps, few, kw, it=8, nslots=2, seed=31)
+    solvers = draw_state(Ps, few, kw, it, nslots, seed=31)
     shapes = {binding.ST_ALPHA: ((DISTINCT, -1), 0), binding.ST_BETA0: ((DISTINCT, -1), 0),
               binding.ST_BETA1: ((DISTINCT, -1), 0), binding.ST_ADAM: ((6, DISTINCT, -1), 1),
               binding.ST_SLOT_ADAM: ((2, DISTINCT, -1), 1), binding.ST_XSNAP: ((DISTINCT, -1), 0),
@@ -82,14 +103,24 @@ def test_windows_of_one_record(name, cap):
         big.set_state(w, rep(few.get_state(w, dt).reshape(shape), axis))
     n0 = lo.shape[1]
     dlo, dhi = (torch.zeros((S, n0), device="cuda") for _ in range(2))
-    big.backward(np.ones(S), None, None, dlo, dhi)
+    dW = [torch.zeros(L["W"].shape, device="cuda") for L in net]
+    big.backward(np.ones(S), dW, None, dlo, dhi)
     dlo, dhi = _firsts(dlo.cpu().numpy()), _firsts(dhi.cpu().numpy())
     bound = _firsts(big.bound(64))
+    refW = [np.zeros(L["W"].shape) for L in net]
     for s, sv in enumerate(solvers):
         g = ev.envelope_gradient(sv.P, sv.st)
         assert bound[s] == pytest.approx(g["value"], abs=1e-4, rel=1e-5)
+        decided = np.abs(du.evaluate(sv.P, sv.st)[1][0]) > 1e-5   # x_0* of the others may be at either end
         for got, ref in ((dlo[s], g["dlo0"]), (dhi[s], g["dhi0"])):
-            np.testing.assert_allclose(got, ref, rtol=1e-4, atol=1e-4 * np.abs(ref).max())
+            np.testing.assert_allclose(got[decided], ref[decided], rtol=1e-4, atol=1e-4 * np.abs(ref).max())
+        copies = len(range(s, S, DISTINCT))
+        for k, L in enumerate(net[:-1], start=1):
+            w = g["dW"][k]
+            refW[k - 1] += copies * (w if L["kind"] == "linear" else ev.filter_gradient(w, sv.P.taps[k], L["W"].shape))
+        refW[-1] += copies * np.outer(C[s], g["dW"][sv.P.n][0])
+    for got, ref in zip(dW, refW):
+        np.testing.assert_allclose(got.cpu().numpy(), ref, rtol=1e-4, atol=1e-4 * np.abs(ref).max())
     big.as_step(1)
     al, b0, b1 = (_firsts(hidden(w)) for w in (binding.ST_ALPHA, binding.ST_BETA0, binding.ST_BETA1))
     sb = _firsts(hidden(binding.ST_SLOT_BETA)).reshape(DISTINCT, big.cap, -1)
