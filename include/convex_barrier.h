@@ -117,14 +117,18 @@ void as_default_options(as_options* opt);
  *              NULL allowed only when n_out == 1 (then C[s] = 1).
  *  lhat, uhat: hidden vectors of pre-activation bounds (App. E), host or device; both NULL
  *              to compute them on the device by interval propagation (App. E, last paragraph),
- *              accumulated in FP64 and rounded outward to float32.
+ *              accumulated to FP64's accuracy and rounded outward to float32.
  *  splits:     hidden vector of int8 ReLU splits (+1 active, -1 inactive, 0 free), or NULL. A
  *              split clamps lhat to 0 (+1) or uhat to 0 (-1) of a neuron whose interval straddles
  *              zero before the next layer is propagated; it is ignored with caller bounds.
  *  caps:       [S] masks per neuron for each subproblem (1..max_cuts), or NULL (= max_cuts).
  *  opt:        NULL for defaults.
  *  stream:     cudaStream_t on which every call of this context is enqueued (NULL = legacy).
- * The context starts with every dual at zero, so its bound is the interval bound (App. B.3). */
+ * The context starts with every dual at zero, so its bound is the interval bound (App. B.3).
+ * A context repeats its results bit for bit. The order of its sums depends on the net and on S (lanes
+ * per neuron; tiles from about 3e7 multiply-adds a pass on), so the same subproblem in a batch of
+ * another size agrees up to float32 rounding, but an input whose f (eq. 7) is within rounding of
+ * zero may take the other end of its box. */
 int as_init(as_ctx** out, const as_net* net, int S, const float* x_lo, const float* x_hi,
             const float* C, const float* lhat, const float* uhat, const signed char* splits,
             const int* caps, const as_options* opt, void* stream);
@@ -231,7 +235,8 @@ long long as_launch_count(as_ctx* ctx);
 #define AS_K_BATCH 12     /* a batch's set-up (as_init, as_reset): box checks, property rows,
                              interval bounds, row constants, fixed inputs                   */
 #define AS_K_SP_START 13  /* Saddle Point's start: statistics (eq. 10), caps (eq. 16), records */
-#define AS_K_COUNTER 14   /* the one-thread launches that advance the iteration counters  */
+#define AS_K_COUNTER 14   /* the one-warp launches that advance the iteration counters and the
+                             schedule                                                       */
 #define AS_K_COUNT 15
 
 /* With as_options.profile set: total device time (CUDA events on the context's stream) and
@@ -250,7 +255,8 @@ const char* as_last_error(as_ctx* ctx);
  * fixed memory pool of a serving engine), where a direct allocation fails or fragments the pool;
  * and latency-critical callers that cannot afford the implicit device synchronisation of
  * cudaMalloc / cudaFree. as_init cannot serve them, since it allocates its context. This entry
- * point computes the pre-activation bounds that as_init derives by interval propagation, with
+ * point computes the pre-activation bounds that as_init derives by interval propagation (bit for
+ * bit those of batches below its tiles' size, up to float32 rounding those of larger ones), with
  * no allocation: the caller passes every input and output, and the post-activation bounds handed
  * from one layer to the next live in a file-scope device array of AS_NOALLOC_SCRATCH_FLOATS
  * floats (16 MiB) that every GPU which loads the library keeps until the process exits.

@@ -1179,7 +1179,7 @@ extern "C" void as_destroy(as_ctx* c) {
 }
 
 // ------------------------------------------------------------------------------- iterations
-// Launches a kernel that begins with cb_after_previous. Where its blocks are at most one per SM, the launch
+// Launches a kernel that begins with cb_after_previous. Where its blocks are at most one per SM (152), the launch
 // overlaps the end of the kernel before it in the stream (programmatic dependent launch). Larger grids launch
 // plainly: blocks that wait take the places of ones that could run, unevenly over the SMs (100 iterations of a
 // three-layer perceptron on one box 1376 -> 1311 us; with every grid so, 25 Saddle Point iterations of the Wide
@@ -1544,7 +1544,7 @@ extern "C" int as_set_state(as_ctx* c, int which, const void* src) {
         if (v[0] < 0 || v[1] < 0) return fail(c, AS_ERR_ARG, "negative iteration counter");
         int w[3] = {v[0], v[1], v[2] ? c->opt.sp_init_steps : 0};
         CUDA_TRY(c, cudaMemcpyAsync(c->st.ctr, w, sizeof w, cudaMemcpyHostToDevice, c->stream));
-    k_set_step<<<1, 32, 0, c->stream>>>(c->st, c->sc);
+        k_set_step<<<1, 32, 0, c->stream>>>(c->st, c->sc);
         CUDA_TRY(c, cudaStreamSynchronize(c->stream));
         c->sp_started = v[2] != 0;
         return recompute_slot_sums(c);

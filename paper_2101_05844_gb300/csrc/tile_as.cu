@@ -153,9 +153,10 @@ struct ColOp : ColRecords<NS> {
 
 // The same sums in the order of a lane per unit (cb_team.cuh): the positive taps of a channel, then its
 // negative ones, into one accumulator of the unmasked product. Two sweeps over the taps for every four
-// channels, for the gradient, whose x* must not depend on which walk found it (an input at a tie of f moves
-// it; the bound is continuous there and takes the packed sums: 16.2 against 8.9 ms at 1024 conv4 boxes and
-// five slots).
+// channels, for the gradient, which an input at a tie of f moves (the bound is continuous there and takes the
+// packed sums: 16.2 against 8.9 ms at 1024 conv4 boxes and five slots). Equal bit for bit to a lane per unit
+// where a tile is not split; a team of several lanes and a split tile add their parts' sums, and an input whose
+// f is within rounding of zero may take its other end there.
 template <int NS, int CH>
 struct ColSeqOp : ColRecords<NS> {
     static constexpr int WB = 4, CW = 4, SWEEPS = 2 * CH / CW;

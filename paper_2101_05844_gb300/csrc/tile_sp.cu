@@ -16,8 +16,8 @@ namespace cb {
 // warp's 32 pairs that meet in float64 (rms over rows of 576 terms 1.1e-15 against 3.4e-16 of the terms'
 // magnitudes). A thread's pair therefore ends where a lane's would, after a 32nd of the row, and goes into a
 // three-word total (CompTotal): no larger error than the warp's at any of 27 to 8192 terms. That costs 20
-// operations per 32nd of a row (4.0 -> 4.7 ms); adding into float64 instead would take about 6 ms on its narrow
-// pipe alone.
+// operations per 32nd of a row (4.0 -> 4.7 ms: of the batch's set-up 3.52 -> 4.14, 3.69 with the totals left out).
+// Adding into float64 instead asks for 4 G conversions and additions, 6 ms at the nominal float64 rate.
 template <int CH>
 struct IbpOp : TlOp {
     static constexpr int RB = 8, EB = 0, WB = 4, SWEEPS = 1;
@@ -483,7 +483,8 @@ void tl_launch_ibp_box(int grid, const DNet& net, const DState& st, cudaStream_t
 
 // Splits of a layer's walks: a layer is one launch, and one with fewer tiles than two per SM (linear layers:
 // 64 at 256 subproblems and 512 rows) leaves most of the chip idle while its blocks walk all their sources. At
-// least 64 taps per split. Without splits 13 conv4 boxes took 1.61 ms, a warp per row 1.53, split 0.60.
+// least 64 taps per split. Without splits 13 conv4 boxes took 1.61 ms, a warp per row 1.53, split 0.60 (one pair a
+// row; the totals changed nothing at this size: the batch's set-up takes 0.54 ms before, 0.53 after).
 int tl_ibp_splits(const TlSeg& g, int S) {
     return std::max(1, std::min({152 * 2 / tl_tiles(g, S), g.nch, 16, g.SC * g.kt / 64}));
 }
